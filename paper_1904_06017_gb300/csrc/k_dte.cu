@@ -2,15 +2,25 @@
 // refinement by gradient (include/stereo_diff.h).
 //
 // Every reduction runs in two fixed-order stages: kDteBlocks blocks per pair write FP64
-// partial sums, one finishing thread per pair adds them in index order.  Per pixel the
-// energy and its adjoint work in FP32 with FP64 accumulation.  The refinement reduces the
-// map once to ten FP64 moments in centred coordinates; every step then evaluates the sums it
-// needs at its angle from them (exact algebra) and solves the normal equations of eq. (alpha3)
-// in FP64.
+// partial sums, one warp per pair adds them.  Per pixel the energy and its adjoint work in
+// FP32; the refinement reduces the map once to ten moments in centred coordinates, and every
+// step evaluates the sums it needs at its angle from them (exact algebra) and the line fit of
+// eq. (alpha3) in FP64.
+//
+// An FP64 instruction of a warp occupies a GB300 SM about 16 times as long as an FP32 one and
+// returns after about 65 cycles, so the per-pixel sums are kept out of FP64: a warp adds its
+// pixels in pairs of floats (the rounding error of every addition and product is recovered
+// exactly and summed beside it, so a sum carries about 48 bits over the thousand or so pixels
+// of a warp) and widens once at the end; sums over pixel coordinates are exact integers.
+// A warp whose pair is not finite (an infinite or NaN disparity, or a sum beyond the FP32
+// range) adds its pixels again in FP64.  8 maps of 960 x 540: energy 13 us (24 us with FP64
+// sums and butterflies), adjoint 18 us (63), moments 22 us (152); all are bound by the FP64
+// tail of a block (the widened warp sums) more than by reading the map.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
 
+#include "dt_trig.cuh"
 #include "internal.cuh"
 #include "stereo_diff.h"
 
@@ -26,28 +36,69 @@ enum { DTE_ENERGY = 0, DTE_BWD = 1 };
 size_t dte_bytes(int B)
 {
     const size_t part = (size_t)B * kDteBlocks * kDteSums * sizeof(double);
-    const size_t state = (size_t)B * 2 * sizeof(double);
-    return (part + 255) / 256 * 256 + (state + 255) / 256 * 256;
+    return (part + 255) / 256 * 256;
 }
 
+// A sum of floats with the rounding errors of its additions beside it.
+struct PairSum {
+    float hi, lo;
+    __device__ __forceinline__ void add(float x)
+    {
+        const float s = __fadd_rn(hi, x), b = __fsub_rn(s, hi);
+        lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(x, b)));
+        hi = s;
+    }
+    // += the exact product x y
+    __device__ __forceinline__ void add_product(float x, float y)
+    {
+        const float p = __fmul_rn(x, y);
+        lo = __fadd_rn(lo, __fmaf_rn(x, y, -p));
+        add(p);
+    }
+    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+    // the total over the 32 lanes of a warp, on every lane
+    __device__ __forceinline__ void warp_add()
+    {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const float h = __shfl_xor_sync(0xffffffffu, hi, o), l = __shfl_xor_sync(0xffffffffu, lo, o);
+            add(h);
+            lo = __fadd_rn(lo, l);
+        }
+    }
+};
+
+// The block's total of every warp's values (lane 0 of each warp holds them), in warp order.
 template <int NS>
-__device__ void block_sum_store(double (&acc)[NS], double *out)
+__device__ void block_sum_store(const double (&acc)[NS], double *out)
 {
     __shared__ double red[kDteThreads / 32][NS];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (lane == 0) {
 #pragma unroll
-    for (int k = 0; k < NS; ++k) {
-        double v = acc[k];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if (lane == 0) red[wid][k] = v;
+        for (int k = 0; k < NS; ++k) red[wid][k] = acc[k];
     }
     __syncthreads();
     if (threadIdx.x < NS) {
         double v = 0.0;
+#pragma unroll
         for (int w = 0; w < kDteThreads / 32; ++w) v += red[w][threadIdx.x];
         out[threadIdx.x] = v;
     }
+}
+
+__device__ __forceinline__ double warp_add(double x)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    return x;
+}
+
+__device__ __forceinline__ long long warp_add(long long x)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    return x;
 }
 
 // Per pixel r = l - alpha0 - alpha1 y(psi), y = v cos(psi) - u sin(psi) (eq. y).
@@ -74,41 +125,94 @@ __global__ void __launch_bounds__(kDteThreads) k_dte(const float *__restrict__ d
     const int HW = W * H;
     const float *L = disp + (size_t)b * HW;
     const uint8_t *M = mask ? mask + (size_t)b * HW : nullptr;
-    double acc[NS];
-#pragma unroll
-    for (int k = 0; k < NS; ++k) acc[k] = 0.0;
-    for (int i = blockIdx.x * kDteThreads + threadIdx.x; i < HW; i += kDteBlocks * kDteThreads) {
+    // the values of pixel i that are summed
+    auto terms = [&](int i, float l, bool in, float (&t)[NS]) {
         const int v = i / W, u = i - v * W;
-        const float m = (!M || M[i]) ? 1.f : 0.f;
+        const float m = in ? 1.f : 0.f;
         const float y = (float)v * c - (float)u * s;
-        const float r = m * (L[i] - a0 - a1 * y);
+        const float r = m * (l - a0 - a1 * y);
         if constexpr (MODE == DTE_ENERGY) {
-            acc[0] += (double)(r * r);
+            t[0] = __fmul_rn(r, r);
         } else {
             if (gdisp) gdisp[(size_t)b * HW + i] = g2 * r;
             const float x = (float)u * c + (float)v * s;
-            acc[0] += (double)(r * x);
-            acc[1] += (double)r;
-            acc[2] += (double)(r * y);
+            t[0] = __fmul_rn(r, x);
+            t[1] = r;
+            t[2] = __fmul_rn(r, y);
         }
+    };
+    constexpr int kStep = kDteBlocks * kDteThreads, kAhead = 4;   // loads in flight per thread
+    const int i0 = blockIdx.x * kDteThreads + threadIdx.x;
+    PairSum ps[NS];
+#pragma unroll
+    for (int k = 0; k < NS; ++k) ps[k] = PairSum{0.f, 0.f};
+    for (int i = i0; i < HW; i += kAhead * kStep) {
+        float l[kAhead];
+        bool in[kAhead];
+#pragma unroll
+        for (int j = 0; j < kAhead; ++j) {
+            const int p = i + j * kStep;
+            l[j] = p < HW ? L[p] : 0.f;
+            in[j] = p < HW && (!M || M[p]);
+        }
+#pragma unroll
+        for (int j = 0; j < kAhead; ++j) {
+            const int p = i + j * kStep;
+            if (p >= HW) break;
+            float t[NS];
+            terms(p, l[j], in[j], t);
+#pragma unroll
+            for (int k = 0; k < NS; ++k) ps[k].add(t[k]);
+        }
+    }
+    double acc[NS];
+    bool finite = true;
+#pragma unroll
+    for (int k = 0; k < NS; ++k) {
+        ps[k].warp_add();
+        finite = finite && isfinite(ps[k].hi) && isfinite(ps[k].lo);
+        acc[k] = ps[k].value();
+    }
+    if (!finite) {   // (the same on every lane)
+#pragma unroll
+        for (int k = 0; k < NS; ++k) acc[k] = 0.0;
+        for (int i = i0; i < HW; i += kStep) {
+            float t[NS];
+            terms(i, L[i], !M || M[i], t);
+#pragma unroll
+            for (int k = 0; k < NS; ++k) acc[k] += (double)t[k];
+        }
+#pragma unroll
+        for (int k = 0; k < NS; ++k) acc[k] = warp_add(acc[k]);
     }
     block_sum_store<NS>(acc, part + ((size_t)b * kDteBlocks + blockIdx.x) * kDteSums);
 }
 
-// One thread per pair adds the partials in block order.
-template <int MODE>
-__global__ void k_dte_finish(const double *__restrict__ part, const double *__restrict__ theta,
-                             const double *__restrict__ gE, double *__restrict__ out, int B)
+// The partials of pair b added by one warp: lane l takes partials l and l + 32, then a
+// butterfly (every lane returns the total).
+template <int NS>
+__device__ __forceinline__ void sum_partials(const double *__restrict__ part, int b, double (&s)[NS])
 {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= B) return;
+    static_assert(kDteBlocks == 64, "two partials per lane");
+    const double *p = part + ((size_t)b * kDteBlocks + (threadIdx.x & 31)) * kDteSums;
+#pragma unroll
+    for (int k = 0; k < NS; ++k) s[k] = p[k] + p[32 * kDteSums + k];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int k = 0; k < NS; ++k) s[k] += __shfl_xor_sync(0xffffffffu, s[k], o);
+}
+
+// One warp (block) per pair.
+template <int MODE>
+__global__ void __launch_bounds__(32) k_dte_finish(const double *__restrict__ part, const double *__restrict__ theta,
+                                                   const double *__restrict__ gE, double *__restrict__ out)
+{
     constexpr int NS = MODE == DTE_ENERGY ? 1 : 3;
+    const int b = blockIdx.x;
     double s[NS];
-#pragma unroll
-    for (int k = 0; k < NS; ++k) s[k] = 0.0;
-    for (int j = 0; j < kDteBlocks; ++j)
-#pragma unroll
-        for (int k = 0; k < NS; ++k) s[k] += part[((size_t)b * kDteBlocks + j) * kDteSums + k];
+    sum_partials<NS>(part, b, s);
+    if (threadIdx.x != 0) return;
     if constexpr (MODE == DTE_ENERGY) {
         out[b] = s[0];
     } else {
@@ -119,9 +223,10 @@ __global__ void k_dte_finish(const double *__restrict__ part, const double *__re
     }
 }
 
-// The ten moments of the fitted pixels in coordinates centred on the image, FP64:
+// The ten moments of the fitted pixels in coordinates centred on the image:
 // n, S_u, S_v, S_l, S_uu, S_uv, S_vv, S_ul, S_vl, S_ll with u' = u - (W-1)/2, v' = v - (H-1)/2.
-// Every sum the refinement needs at an angle psi is a fixed combination of them.
+// Every sum the refinement needs at an angle psi is a fixed combination of them.  The
+// coordinates enter doubled (whole numbers); the sums with l are pair sums of exact products.
 __global__ void __launch_bounds__(kDteThreads) k_dref_moments(const float *__restrict__ disp,
                                                               const uint8_t *__restrict__ mask,
                                                               double *__restrict__ part, int W, int H)
@@ -130,24 +235,60 @@ __global__ void __launch_bounds__(kDteThreads) k_dref_moments(const float *__res
     const int HW = W * H;
     const float *L = disp + (size_t)b * HW;
     const uint8_t *M = mask ? mask + (size_t)b * HW : nullptr;
-    const double uc = 0.5 * (W - 1), vc = 0.5 * (H - 1);
-    double acc[kDteSums];
+    constexpr int kStep = kDteBlocks * kDteThreads, kAhead = 4;
+    const int i0 = blockIdx.x * kDteThreads + threadIdx.x;
+    int n = 0;
+    long long su = 0, sv = 0, suu = 0, suv = 0, svv = 0;   // sums over 2u', 2v' and their products
+    PairSum sl{0.f, 0.f}, sul{0.f, 0.f}, svl{0.f, 0.f}, sll{0.f, 0.f};
+    for (int i = i0; i < HW; i += kAhead * kStep) {
+        float l[kAhead];
+        bool in[kAhead];
 #pragma unroll
-    for (int k = 0; k < kDteSums; ++k) acc[k] = 0.0;
-    for (int i = blockIdx.x * kDteThreads + threadIdx.x; i < HW; i += kDteBlocks * kDteThreads) {
-        if (M && !M[i]) continue;
-        const int v = i / W, u = i - v * W;
-        const double x = (double)u - uc, y = (double)v - vc, l = (double)L[i];
-        acc[0] += 1.0;
-        acc[1] += x;
-        acc[2] += y;
-        acc[3] += l;
-        acc[4] = fma(x, x, acc[4]);
-        acc[5] = fma(x, y, acc[5]);
-        acc[6] = fma(y, y, acc[6]);
-        acc[7] = fma(x, l, acc[7]);
-        acc[8] = fma(y, l, acc[8]);
-        acc[9] = fma(l, l, acc[9]);
+        for (int j = 0; j < kAhead; ++j) {
+            const int p = i + j * kStep;
+            l[j] = p < HW ? L[p] : 0.f;
+            in[j] = p < HW && (!M || M[p]);
+        }
+#pragma unroll
+        for (int j = 0; j < kAhead; ++j) {
+            if (!in[j]) continue;
+            const int p = i + j * kStep, v = p / W, u = p - v * W;
+            const int x = 2 * u - (W - 1), y = 2 * v - (H - 1);
+            ++n;
+            su += x;
+            sv += y;
+            suu += (long long)x * x;
+            suv += (long long)x * y;
+            svv += (long long)y * y;
+            sl.add(l[j]);
+            sul.add_product(0.5f * (float)x, l[j]);
+            svl.add_product(0.5f * (float)y, l[j]);
+            sll.add_product(l[j], l[j]);
+        }
+    }
+    sl.warp_add();
+    sul.warp_add();
+    svl.warp_add();
+    sll.warp_add();
+    n = __reduce_add_sync(0xffffffffu, n);
+    double acc[kDteSums] = {(double)n, 0.5 * (double)warp_add(su), 0.5 * (double)warp_add(sv), sl.value(),
+                            0.25 * (double)warp_add(suu), 0.25 * (double)warp_add(suv), 0.25 * (double)warp_add(svv),
+                            sul.value(), svl.value(), sll.value()};
+    if (!(isfinite(acc[3]) && isfinite(acc[7]) && isfinite(acc[8]) && isfinite(acc[9]))) {   // (the same on every lane)
+        double f[4] = {0.0, 0.0, 0.0, 0.0};
+        for (int i = i0; i < HW; i += kStep) {
+            if (M && !M[i]) continue;
+            const int v = i / W, u = i - v * W;
+            const double x = (double)u - 0.5 * (W - 1), y = (double)v - 0.5 * (H - 1), l = (double)L[i];
+            f[0] += l;
+            f[1] = fma(x, l, f[1]);
+            f[2] = fma(y, l, f[2]);
+            f[3] = fma(l, l, f[3]);
+        }
+        acc[3] = warp_add(f[0]);
+        acc[7] = warp_add(f[1]);
+        acc[8] = warp_add(f[2]);
+        acc[9] = warp_add(f[3]);
     }
     block_sum_store<kDteSums>(acc, part + ((size_t)b * kDteBlocks + blockIdx.x) * kDteSums);
 }
@@ -160,66 +301,81 @@ __device__ double wrap_half_pi_d(double psi)
     return psi;
 }
 
-// All refinement steps of one pair (one thread per pair).  At each angle the sums over the
-// fitted pixels of y, y^2, l y, x, x y, x^2, l x (raw coordinates, x = u cos + v sin, y = v cos
-// - u sin, eq. x, eq. y) follow from the centred moments; then the line fit of eq. (alpha3)
-// from the FP64 normal equations, E and g = dE/dpsi there (eq. d_e_min), the Gauss-Newton
-// curvature and the step psi <- wrap(psi - g / H).  Trajectory entry k is written at each step.
-__global__ void k_dref_run(const double *__restrict__ part, const double *__restrict__ state, double *__restrict__ traj,
-                           int steps, int W, int H, int B)
+// All refinement steps of one pair (one warp per pair).  The moments, per pixel and about the
+// centroid of the fitted pixels, are taken once; at an angle, with x = u cos + v sin and
+// y = v cos - u sin (eq. x, eq. y), the line fit of eq. (alpha3) is alpha1 = C_yl / C_yy and
+// alpha0 = mean(l) - alpha1 mean(y), E = n (C_ll - alpha1 C_yl), g = dE/dpsi = 2 n alpha1
+// (C_xl - alpha1 C_xy) (eq. d_e_min), and the Gauss-Newton curvature H = 2 n alpha1^2
+// (C_xx - C_xy^2 / C_yy); the step is psi <- wrap(psi - g / H).
+//
+// The steps are one FP64 dependency chain, so only what the next angle needs is on it: with
+// C_xx C_yy - C_xy^2 = det, the same at every angle, g / H = C_yy (C_xl C_yy - C_yl C_xy) /
+// (C_yl det), one quotient.  Its reciprocal is an FP32 one with one Newton step in FP64 (about
+// 47 bits: an error of 1e-14 of the step, which the next step corrects), or the full division
+// where FP32 cannot hold the divisor.  The angles go to shared memory, and the trajectory's
+// entries are then evaluated with one step per lane.  50 steps: 102 us (289 us with the sums
+// over raw coordinates and every quantity of a step evaluated on the chain).
+constexpr int kDrefSteps = 1000;   // the most steps a call may ask for
+
+__global__ void __launch_bounds__(32) k_dref_run(const double *__restrict__ part, double psi_init,
+                                                 double *__restrict__ traj, int steps, int W, int H)
 {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= B) return;
+    __shared__ double sp[kDrefSteps + 1];
+    const int b = blockIdx.x;
     double m[kDteSums];
-    for (int q = 0; q < kDteSums; ++q) m[q] = 0.0;
-    for (int j = 0; j < kDteBlocks; ++j)
-        for (int q = 0; q < kDteSums; ++q) m[q] += part[((size_t)b * kDteBlocks + j) * kDteSums + q];
-    const double n = m[0], Su = m[1], Sv = m[2], Sl = m[3], Suu = m[4], Suv = m[5], Svv = m[6], Sul = m[7],
-                 Svl = m[8], Sll = m[9];
-    const double uc = 0.5 * (W - 1), vc = 0.5 * (H - 1);
-    double psi = state[2 * b];
-    for (int k = 0; k <= steps; ++k) {
-        const double c = cos(psi), s = sin(psi);
-        // raw x = x' + xc, y = y' + yc with the centred rotated coordinates x', y'
-        const double xc = uc * c + vc * s, yc = vc * c - uc * s;
-        const double Sx1 = Su * c + Sv * s, Sy1 = Sv * c - Su * s;                // sums of x', y'
-        const double Sxx1 = c * c * Suu + 2.0 * c * s * Suv + s * s * Svv;
-        const double Syy1 = c * c * Svv - 2.0 * c * s * Suv + s * s * Suu;
-        const double Sxy1 = c * s * (Svv - Suu) + (c * c - s * s) * Suv;
-        const double Slx1 = Sul * c + Svl * s, Sly1 = Svl * c - Sul * s;
-        const double Sy = Sy1 + n * yc, Sx = Sx1 + n * xc;
-        const double Syy = Syy1 + 2.0 * yc * Sy1 + n * yc * yc;
-        const double Sxx = Sxx1 + 2.0 * xc * Sx1 + n * xc * xc;
-        const double Sxy = Sxy1 + xc * Sy1 + yc * Sx1 + n * xc * yc;
-        const double Sly = Sly1 + yc * Sl, Slx = Slx1 + xc * Sl;
-        const double det = n * Syy - Sy * Sy;
-        double a0 = 0.0, a1 = 0.0, g = 0.0, Hc = 0.0;
-        if (n > 0.0 && det > 0.0) {
-            a0 = (Syy * Sl - Sy * Sly) / det;
-            a1 = (n * Sly - Sy * Sl) / det;
-            g = 2.0 * a1 * (Slx - a0 * Sx - a1 * Sxy);
-            const double xt2 = Sxx - (Syy * Sx * Sx - 2.0 * Sy * Sx * Sxy + n * Sxy * Sxy) / det;
-            Hc = 2.0 * a1 * a1 * xt2;
-        } else if (n > 0.0) {
-            a0 = Sl / n;
+    sum_partials<kDteSums>(part, b, m);
+    // (divisions: the mean of equal coordinates is that coordinate exactly, and its spread 0)
+    const double n = m[0], n1 = n > 0.0 ? n : 1.0;
+    const double mu = m[1] / n1, mv = m[2] / n1, ml = m[3] / n1;
+    const double Cuu = (m[4] - m[1] * mu) / n1, Cuv = (m[5] - m[1] * mv) / n1, Cvv = (m[6] - m[2] * mv) / n1;
+    const double Cul = (m[7] - m[1] * ml) / n1, Cvl = (m[8] - m[2] * ml) / n1, Cll = (m[9] - m[3] * ml) / n1;
+    const double Cdf = Cvv - Cuu, det = Cuu * Cvv - Cuv * Cuv;
+    double psi = wrap_half_pi_d(psi_init);
+    for (int k = 0; k < steps; ++k) {
+        if (threadIdx.x == 0) sp[k] = psi;
+        double s, c;
+        sincos_half_pi(psi, &s, &c);
+        const double cs = c * s, ss = s * s;
+        const double Cyy = (Cvv - ss * Cdf) - 2.0 * cs * Cuv, Cxy = cs * Cdf + (Cuv - 2.0 * ss * Cuv);
+        const double Cyl = c * Cvl - s * Cul, Cxl = c * Cul + s * Cvl;
+        if (!(Cyy > 0.0)) continue;   // no line to fit: the angle stays
+        const double num = Cyy * (Cxl * Cyy - Cyl * Cxy), den = Cyl * det;
+        const float r0 = 1.0f / (float)den;
+        double d;
+        if (fabsf(r0) > 1e-30f && fabsf(r0) < 1e30f) {
+            const double r = (double)r0;
+            d = num * (r * (2.0 - den * r));
+        } else {
+            d = num / den;
         }
-        const double E = Sll - 2.0 * a0 * Sl - 2.0 * a1 * Sly + a0 * a0 * n + 2.0 * a0 * a1 * Sy + a1 * a1 * Syy;
+        // a step only where the curvature is positive (C_yl^2 det > 0) and the quotient finite
+        if (den * Cyl > 0.0 && isfinite(d)) {
+            psi -= d;
+            if (psi > 0.5 * M_PI || psi <= -0.5 * M_PI) psi = wrap_half_pi_d(psi);
+        }
+    }
+    if (threadIdx.x == 0) sp[steps] = psi;
+    __syncwarp();
+    const double uc = mu + 0.5 * (W - 1), vc = mv + 0.5 * (H - 1);   // the centroid in raw coordinates
+    for (int k = threadIdx.x; k <= steps; k += 32) {
+        const double p = sp[k];
+        double s, c;
+        sincos_half_pi(p, &s, &c);
+        const double cs = c * s, ss = s * s;
+        const double Cyy = (Cvv - ss * Cdf) - 2.0 * cs * Cuv, Cxy = cs * Cdf + (Cuv - 2.0 * ss * Cuv);
+        const double Cyl = c * Cvl - s * Cul, Cxl = c * Cul + s * Cvl;
+        double a0 = ml, a1 = 0.0, g = 0.0;
+        if (n > 0.0 && Cyy > 0.0) {
+            a1 = Cyl / Cyy;
+            g = 2.0 * n * a1 * (Cxl - a1 * Cxy);
+            a0 = ml - a1 * (vc * c - uc * s);
+        }
         double *t = traj + ((size_t)b * (steps + 1) + k) * 5;
-        t[0] = psi;
+        t[0] = p;
         t[1] = a0;
         t[2] = a1;
         t[3] = g;
-        t[4] = E;
-        if (k < steps && Hc > 0.0 && isfinite(g / Hc)) psi = wrap_half_pi_d(psi - g / Hc);
-    }
-}
-
-__global__ void k_dref_init(double *state, double psi, int B)
-{
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b < B) {
-        state[2 * b] = wrap_half_pi_d(psi);
-        state[2 * b + 1] = 0.0;
+        t[4] = n * (Cll - a1 * Cyl);
     }
 }
 
@@ -238,12 +394,6 @@ int check_dte_ws(int B, void *ws, size_t bytes, const char *who)
     if (bytes < dte_bytes(B))
         return set_error(STEREO_EINVAL, "%s: workspace of %zu bytes, %zu needed", who, bytes, dte_bytes(B));
     return STEREO_OK;
-}
-
-double *dte_state(int B, void *ws)
-{
-    const size_t part = (size_t)B * kDteBlocks * kDteSums * sizeof(double);
-    return (double *)((char *)ws + (part + 255) / 256 * 256);
 }
 
 }  // namespace
@@ -272,7 +422,7 @@ extern "C" int stereo_dt_energy_fwd(int32_t W, int32_t H, int32_t B, const float
     double *part = (double *)ws;
     k_dte<DTE_ENERGY><<<dim3(kDteBlocks, B), kDteThreads, 0, st>>>(disp, mask, theta, nullptr, nullptr, part,
                                                                     W, H);
-    k_dte_finish<DTE_ENERGY><<<(B + 63) / 64, 64, 0, st>>>(part, theta, nullptr, energy, B);
+    k_dte_finish<DTE_ENERGY><<<B, 32, 0, st>>>(part, theta, nullptr, energy);
     return cuda_error(cudaGetLastError(), who);
 }
 
@@ -289,7 +439,7 @@ extern "C" int stereo_dt_energy_bwd(int32_t W, int32_t H, int32_t B, const float
     cudaStream_t st = (cudaStream_t)stream;
     double *part = (double *)ws;
     k_dte<DTE_BWD><<<dim3(kDteBlocks, B), kDteThreads, 0, st>>>(disp, mask, theta, gE, gdisp, part, W, H);
-    if (gtheta) k_dte_finish<DTE_BWD><<<(B + 63) / 64, 64, 0, st>>>(part, theta, gE, gtheta, B);
+    if (gtheta) k_dte_finish<DTE_BWD><<<B, 32, 0, st>>>(part, theta, gE, gtheta);
     return cuda_error(cudaGetLastError(), who);
 }
 
@@ -301,13 +451,12 @@ extern "C" int stereo_dt_refine_roll(int32_t W, int32_t H, int32_t B, const floa
     int rc = check_sizes(W, H, B, who);
     if (rc) return rc;
     if (!disp || !traj) return set_error(STEREO_EINVAL, "%s: null pointer", who);
-    if (steps < 0 || steps > 1000) return set_error(STEREO_EINVAL, "%s: steps %d outside 0..1000", who, steps);
+    if (steps < 0 || steps > kDrefSteps) return set_error(STEREO_EINVAL, "%s: steps %d outside 0..%d", who, steps, kDrefSteps);
     if (!isfinite(psi_init)) return set_error(STEREO_EINVAL, "%s: psi_init not finite", who);
     if ((rc = check_dte_ws(B, ws, ws_bytes, who))) return rc;
     cudaStream_t st = (cudaStream_t)stream;
-    double *part = (double *)ws, *state = dte_state(B, ws);
-    k_dref_init<<<(B + 63) / 64, 64, 0, st>>>(state, psi_init, B);
+    double *part = (double *)ws;
     k_dref_moments<<<dim3(kDteBlocks, B), kDteThreads, 0, st>>>(disp, mask, part, W, H);
-    k_dref_run<<<(B + 63) / 64, 64, 0, st>>>(part, state, traj, steps, W, H, B);
+    k_dref_run<<<B, 32, 0, st>>>(part, psi_init, traj, steps, W, H);
     return cuda_error(cudaGetLastError(), who);
 }

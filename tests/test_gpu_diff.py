@@ -392,3 +392,27 @@ def test_warp_coefficients_refined_through_autograd(scene):
     h = 1e-3
     fd0 = (loss(c0_0 + h, c1_0) - loss(c0_0 - h, c1_0)) / (2 * h)
     assert go[0] == pytest.approx(fd0, rel=1e-3)
+
+
+@pytest.mark.parametrize("H,W,value", [(1, 1, 3.0), (1, 9, 3.0), (9, 1, 3.0), (130, 131, 3.0), (40, 50, np.inf),
+                                       (40, 50, np.nan), (40, 50, 3e19)])
+def test_energy_and_refinement_sums_at_their_edges(H, W, value):
+    """Maps of one row, one column, one pixel, and maps holding an infinity, a NaN or a value
+    whose square leaves the FP32 range: eq. (E2) within 1e-5 of its FP64 sum (FP32 residuals), the
+    same infinity or NaN where the sum has one, and the moments' constant map fitted exactly."""
+    rng = np.random.default_rng(H * W)
+    d = (5.0 + 0.1 * np.arange(H)[:, None] + 0.02 * rng.standard_normal((H, W))).astype(np.float32)
+    d[H // 2, W // 2] = value
+    theta = torch.tensor([[0.02, 4.0, 0.09]], dtype=torch.float64, device="cuda")
+    e = sgd.dt_energy(dev(d)[None], theta)
+    u, v = np.meshgrid(np.arange(W, dtype=np.float64), np.arange(H, dtype=np.float64))
+    with np.errstate(over="ignore", invalid="ignore"):
+        r = (d.astype(np.float64) - 4.0 - 0.09 * (v * math.cos(0.02) - u * math.sin(0.02)))
+        want = np.sum((r * r).astype(np.float32).astype(np.float64))
+    got = float(e[0])
+    if np.isfinite(want):
+        assert abs(got - want) <= 1e-5 * max(want, 1.0)
+    else:
+        assert got == want or (math.isnan(got) and math.isnan(want))
+    flat = sgd.refine_roll(torch.full((1, H, W), 2.5, device="cuda"), None, 0.1, 3).cpu().numpy()[0]
+    assert np.allclose(flat[:, 0], 0.1) and np.allclose(flat[:, 1], 2.5, atol=1e-9) and np.allclose(flat[:, 2:], 0, atol=1e-6)
