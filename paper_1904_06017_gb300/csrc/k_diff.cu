@@ -15,13 +15,19 @@
 //   k_dagg<GC>  gc(q,d) = sum_p w(p,q) h(p,d)                  (adjoint of eq. fbs in c)
 //               gw(x) = 2/sigma1^2 (t1(x) + sum_d c(x,d) sum_q w (I_q - I_x) h(q,d)
 //                                        - sum_q w (I_q - I_x) beta(q))  (through the weights)
-//   k_dcost_bwd adjoint of eq. (c): with A = -gc/(n s_a s_b), B = gc ncc/(n s_a^2),
-//               C = gc ncc/(n s_b^2) per window pair, every extended reference position X
-//               collects  sum_d sum_q A (t - mu_b) + B (r - mu_a)            -> gref_ext(X)
-//               and for the target position X - d:  sum_q A (r - mu_a) + C (t - mu_b) -> Gamma(X,d),
-//               summed over d per X - d inside each tile (partial diagonal sums; Gamma itself
-//               is never stored)
-//   k_dtgt_diag gtw_ext(Xt) = sum_d Gamma(Xt + d, d): the tiles' partial sums added
+//   k_dcost_bwd adjoint of eq. (c).  Per window pair (q, d), with g = gc(q,d) / n and the target
+//               block qt = q - d:  A = -g / (s_a s_b),  B = g ncc / s_a^2,  C = g ncc / s_b^2;
+//               an extended reference position X collects
+//                   sum_d sum_q A (t(X-d) - mu_b(qt)) + B (r(X) - mu_a(q))
+//               and a target position Xt, with X = Xt + d,
+//                   sum_d sum_q A (r(X) - mu_a(q)) + C (t(Xt) - mu_b(qt)),
+//               q over the window of X.  Only A meets a value that changes with both X and d, so
+//               only A is summed over the window for every d (bA); everything else is summed over
+//               d first, along q (reference) or along qt (target), and over the window once:
+//                   gref(X)  = sum_d t(X-d) bA(X,d) + box(-sum_d A mu_b - mu_a sum_d B) + r(X) box(sum_d B)
+//                   gtw(Xt)  = sum_d r(X) bA(X,d) + box(-sum_d A mu_a - mu_b sum_d C) + t(Xt) box(sum_d C)
+//               (every tile writes partial sums over its columns of what runs along Xt or qt)
+//   k_dbox      adds the tiles' partial sums and the window sums of both sides
 //   k_dfold     fold the clamp-to-edge positions back onto the image and undo the warp
 #include <cuda_runtime.h>
 #include <math.h>
@@ -58,8 +64,8 @@ constexpr int kCostDC = 16;          // disparities per block in k_dcost
 constexpr float kFar = 1e18f;        // scaled intensity of an out-of-image neighbour: weight 0
 constexpr float kLog2e = 1.4426950408889634f;
 
-// The cost adjoint's tiles are 32 extended columns wide; each sums Gamma(X, d) over d into
-// 32 + D - 1 entries per row, one per target column X - d its columns reach.
+// The cost adjoint's tiles are 32 extended columns wide; each sums what runs along X - d or q - d
+// into 32 + D - 1 entries per row, one per target column its columns reach.
 __host__ __device__ constexpr int cb_tiles_x(int Wr) { return (Wr + 31) / 32; }
 __host__ __device__ constexpr int cb_diag_w(int D) { return 32 + D - 1; }
 
@@ -97,7 +103,7 @@ struct Dims {
 
 struct Ws {
     float *tw, *mur, *sdr, *mut, *isdt, *cost, *lse, *lbar;      // forward (isdt: 1 / s_b, 0 where flat)
-    float *h, *gc, *beta, *t1, *gw, *gpart, *grefx, *gtwx;      // backward
+    float *h, *gc, *beta, *t1, *gw, *gpart, *gqpart, *samb, *sb, *grefx, *gtwx;      // backward
 };
 
 size_t layout(const Dims &d, char *base, Ws *w)
@@ -124,6 +130,9 @@ size_t layout(const Dims &d, char *base, Ws *w)
     take(&o->t1, B * img);
     take(&o->gw, B * img);
     take(&o->gpart, B * (size_t)d.Hr * cb_tiles_x(d.Wr) * cb_diag_w(d.D));
+    take(&o->gqpart, 2 * B * (size_t)d.H * cb_tiles_x(d.Wr) * cb_diag_w(d.D));
+    take(&o->samb, B * img);
+    take(&o->sb, B * img);
     take(&o->grefx, B * (size_t)d.Hr * d.Wr);
     take(&o->gtwx, B * (size_t)d.Hr * d.Wt);
     return off;
@@ -784,74 +793,80 @@ __global__ void __launch_bounds__(agg_threads(MODE), MODE == AGG_FWD ? 3 : MODE 
 // ------------------------------------------------------------------ cost adjoint
 struct CbArgs {
     const float *ref, *tw, *mur, *sdr, *mut, *isdt, *cost, *gc;
-    float *gpart;          // [B][Hr][tile column][32 + D - 1] partial diagonal sums of Gamma (or null)
-    float *grefx;
+    float *gpart;          // [B][Hr][tile column][32 + D - 1] partial sums over X of r(X) bA(X, d) (or null)
+    float2 *gqpart;        // [B][H][tile column][32 + D - 1] partial sums over q of (A mu_a, C) (or null)
+    float *samb, *sb;      // [B][H][W] sum_d A mu_b, sum_d B
+    float *grefx;          // [B][Hr][Wr] sum_d t(X-d) bA(X, d)
     int W, H, D, Wr, Hr, We;
     float inv_n;
 };
 
-// Extended reference positions X in [-rw, W-1+rw] x [-rw, H-1+rw], a 32 x kCbTY tile per block
-// (a thread owns two of its rows, 8 apart).
-// kCbDC disparities at a time: the four window-pair terms A, A mu_a, C, C mu_b of the pairs q
-// in the tile's halo are staged and box-summed with running sums (along rows, then along
-// columns); the d-independent terms of the reference gradient are summed over d per q and
-// box-summed once at the end.  Row strides are padded to odd lengths so that the running
-// sums of neighbouring rows hit distinct shared-memory banks.  Gamma(X, d) is added into a
-// shared row per tile row at entry X - X0 - d + D - 1 (within one step of d every lane of a
-// warp meets a distinct entry; the two steps of a round are ordered by a warp barrier, the
-// rounds by the block's), and the tile's rows of partial sums are written once at the end.
-constexpr int kCbDC = 2;
-constexpr int kCbTY = 16;   // extended rows per tile (two per thread, 8 apart)
-
-// Running box sums of one half of a plane row: out[x] = sum_{j < WN} in[x + j], x < 16.
-template <int WN>
-__device__ __forceinline__ void row_box16(const float *in, float *out)
+// The constants that are subtracted from the reference values and means (x) and the target's
+// (y): both adjoints depend only on differences t - mu_b and r - mu_a, which are here formed
+// after sums over d, so the images' common level is taken off first.  The median of three
+// pixels (0 where it is not finite).
+__device__ __forceinline__ float median3(float a, float b, float c)
 {
-    float s = 0.f;
-#pragma unroll
-    for (int j = 0; j < WN; ++j) s += in[j];
-    out[0] = s;
-#pragma unroll
-    for (int x = 1; x < 16; ++x) {
-        s += in[x + WN - 1] - in[x - 1];
-        out[x] = s;
-    }
+    const float m = fmaxf(fminf(a, b), fminf(fmaxf(a, b), c));
+    return isfinite(m) ? m : 0.f;
+}
+__device__ __forceinline__ float2 cb_levels(const float *ref, const float *tw, int W, int H)
+{
+    const size_t p0 = (size_t)(H / 2) * W + W / 2, p1 = (size_t)(H / 4) * W + W / 4, p2 = (size_t)(3 * H / 4) * W + 3 * W / 4;
+    return make_float2(median3(ref[p0], ref[p1], ref[p2]), median3(tw[p0], tw[p1], tw[p2]));
 }
 
-// Running box sums of one plane row: out[x] = sum_{j < WN} in[x + j], x < 32.
-template <int WN>
-__device__ __forceinline__ void row_box(const float *in, float *out)
-{
-    float s = 0.f;
-#pragma unroll
-    for (int j = 0; j < WN; ++j) s += in[j];
-    out[0] = s;
-#pragma unroll 8
-    for (int x = 1; x < 32; ++x) {
-        s += in[x + WN - 1] - in[x - 1];
-        out[x] = s;
-    }
-}
+// Extended reference positions X in [-rw, W-1+rw] x [-rw, H-1+rw], a 32 x cb_ty tile per block
+// (a thread owns cb_ty / 8 of its rows, 8 apart).
+// kCbDC disparities at a time: A of the pairs q in the tile's halo is staged and box-summed with
+// running sums (along rows, then along columns).  The pairs q of the tile itself (the halo
+// region's first 32 columns and cb_ty rows: the tiles' own pairs cover the image once) also add
+// up their sums over d.  Row strides are padded to odd lengths so that the running sums of
+// neighbouring rows hit distinct shared-memory banks.  What runs along X - d or q - d is added
+// into shared rows at entry (column in tile) - d + D - 1 (within one step of d every lane of a
+// warp meets a distinct entry, and a row belongs to one warp; the steps of a round are ordered
+// by a warp barrier), and the tile's rows of partial sums are written once at the end.
+// One plane per disparity instead of four (A, A mu_a, C, C mu_b), so a round takes four
+// disparities where it took two.  The bound is latency and the LSU pipe (staged loads, box
+// sums).  8 x 960 x 540, D = 64, w = 9: 1.57 ms and 0.16 ms in k_dbox (2.70 ms with four planes).
+constexpr int kCbDC = 4;
+// extended rows per tile: 24 while a thread's share of the halo (5 pairs) fits its registers
+__host__ __device__ constexpr int cb_ty(int rw) { return rw <= 4 ? 24 : 16; }
+
+template <int RW>
+struct CbShape {
+    static constexpr int TY = cb_ty(RW), QW = 32 + 2 * RW, QH = TY + 2 * RW, NQ = QW * QH, SW = QW | 1;
+    static constexpr size_t planes = (size_t)kCbDC * (SW * QH + 33 * QH + TY * 32);   // floats
+    static size_t smem(int D) { return (planes + (size_t)4 * TY * cb_diag_w(D)) * sizeof(float); }
+};
 
 template <int RW>
 __global__ void __launch_bounds__(256, 2) k_dcost_bwd(const CbArgs a)
 {
-    constexpr int TY = kCbTY, RPT = TY / 8;                     // tile rows; rows per thread (8 apart)
-    constexpr int QW = 32 + 2 * RW, QH = TY + 2 * RW, NQ = QW * QH, NS = (NQ + 255) / 256;
-    constexpr int WN = 2 * RW + 1, DC = kCbDC, NP = 4 * DC;   // planes: 4 terms x DC disparities
-    constexpr int SW = QW | 1, SP = SW * QH;                    // staged row stride (odd), plane size
+    using S = CbShape<RW>;
+    constexpr int TY = S::TY, RPT = TY / 8;                     // tile rows; rows per thread (8 apart)
+    constexpr int QH = S::QH, NQ = S::NQ, NS = (NQ + 255) / 256;
+    constexpr int NO = TY * 32 / 256;                           // a thread's first NO pairs are the tile's own
+    constexpr int WN = 2 * RW + 1, DC = kCbDC;
+    constexpr int SW = S::SW, SP = SW * QH;                     // staged row stride (odd), plane size
     constexpr int HW_ = 33, HP = HW_ * QH;                      // row-summed row stride (odd), plane size
     extern __shared__ float cb_smem[];
-    float *st = cb_smem;                       // [NP][QH][SW]
-    float *hb = st + NP * SP;                  // [NP][QH][33]
-    float *vb = hb + NP * HP;                  // [NP][TY][32]
-    float *gts = vb + NP * TY * 32;            // [TY][32 + D - 1] partial diagonal sums
+    const int GW = cb_diag_w(a.D);
+    float2 *gq = reinterpret_cast<float2 *>(cb_smem);           // [TY][GW] sums of (A mu_a, C) along q - d
+    float *gts = reinterpret_cast<float *>(gq + TY * GW);       // [TY][GW] sums of r bA along X - d
+    float *tr = gts + TY * GW;                                  // [TY][GW] t(X - d) of the tile's rows
+    float *st = tr + TY * GW;                                   // [DC][QH][SW] A
+    float *hb = st + DC * SP;                                   // [DC][QH][33]
+    float *vb = hb + DC * HP;                                   // [DC][TY][32]
     const int b = blockIdx.z;
     const int W = a.W, H = a.H, D = a.D;
     const size_t HW = (size_t)H * W;
     const int X0 = blockIdx.x * 32 - RW, Y0 = blockIdx.y * TY - RW;   // image coords of the tile origin
-    float qmu[NS], qisa[NS], sAmb[NS], sB[NS], sBmu[NS];
-    size_t vbase[NS], sbase[NS];       // cost / gc entry of (q, d = 0); statistics entry of (q, 0)
+    const float *refb = a.ref + b * HW, *twb = a.tw + b * HW;
+    const float2 lev = cb_levels(refb, twb, W, H);
+    const bool tgt = a.gpart != nullptr;
+    float qmu[NO], qisa[NS], sAmb[NO], sB[NO];
+    int qo[NS], so[NS];                // offsets of q in an image and in the target statistics (d = 0)
     int qofs[NS];                      // q's offset inside a staged plane
     bool qin[NS];
     // The halo's pairs q are taken in 32-column slabs (a warp's lanes on one staged row of the
@@ -871,232 +886,333 @@ __global__ void __launch_bounds__(256, 2) k_dcost_bwd(const CbArgs a)
         const int qy = Y0 - RW + r, qx = X0 - RW + c;
         qin[s] = j < NQ && qy >= 0 && qy < H && qx >= 0 && qx < W;
         qofs[s] = j < NQ ? r * SW + c : 0;
-        const size_t qo = qin[s] ? (size_t)qy * W + qx : 0;
-        vbase[s] = (size_t)b * D * HW + qo;
-        sbase[s] = qin[s] ? ((size_t)b * H + qy) * a.We + qx + D - 1 : 0;
-        qmu[s] = qin[s] ? a.mur[b * HW + qo] : 0.f;
-        const float sa = qin[s] ? a.sdr[b * HW + qo] : 0.f;
+        qo[s] = qin[s] ? qy * W + qx : 0;
+        so[s] = qin[s] ? qy * a.We + qx + D - 1 : D - 1;
+        const float sa = qin[s] ? a.sdr[b * HW + qo[s]] : 0.f;
         qisa[s] = sa > 0.f ? __frcp_rn(sa) : 0.f;       // 0 marks a flat reference block
-        sAmb[s] = sB[s] = sBmu[s] = 0.f;
+        if (s < NO) {
+            qmu[s] = qin[s] ? a.mur[b * HW + qo[s]] - lev.x : 0.f;
+            sAmb[s] = sB[s] = 0.f;
+        }
     }
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int X = X0 + tx;
     float rv[RPT], gacc[RPT];
     bool xin[RPT];
-    const float *twrow[RPT];
 #pragma unroll
     for (int i = 0; i < RPT; ++i) {
         const int Y = Y0 + ty + 8 * i;
         xin[i] = X <= W - 1 + RW && Y <= H - 1 + RW;
-        const int yc = clampi(Y, 0, H - 1);
-        rv[i] = a.ref[b * HW + (size_t)yc * W + clampi(X, 0, W - 1)];
-        twrow[i] = a.tw + b * HW + (size_t)yc * W;
+        rv[i] = refb[(size_t)clampi(Y, 0, H - 1) * W + clampi(X, 0, W - 1)] - lev.x;
         gacc[i] = 0.f;
     }
-    const int GW = cb_diag_w(D);
-    if (a.gpart)
-        for (int i = threadIdx.x; i < TY * GW; i += 256) gts[i] = 0.f;   // (the first round's barriers order these)
+    for (int i = threadIdx.x; i < TY * GW; i += 256) {   // (the first round's barriers order these)
+        const int r = i / GW, j = i - r * GW;
+        gq[i] = make_float2(0.f, 0.f);
+        gts[i] = 0.f;
+        tr[i] = twb[(size_t)clampi(Y0 + r, 0, H - 1) * W + clampi(X0 + j - (D - 1), 0, W - 1)] - lev.y;
+    }
     // the loads of a round are issued one round ahead, so that they are in flight while the
     // previous round's box sums run
-    float g[NS][DC], cc[NS][DC], sb[NS][DC], mb[NS][DC];
-    // the target values t(X - d) of the tile rows, loaded a round ahead too (but for the widest
-    // window, whose registers they would spill)
-    constexpr bool TPF = RW < 7;
-    float tn[RPT][DC];
+    const float *gcb = a.gc + (size_t)b * D * HW, *cob = a.cost + (size_t)b * D * HW;
+    const float *isb = a.isdt + (size_t)b * H * a.We, *mub = a.mut + (size_t)b * H * a.We;
+    float g[NS][DC], sbv[NS][DC], cc[NO][DC], mb[NO][DC];
     auto load_round = [&](int d0) {
-        if constexpr (TPF) {
 #pragma unroll
-            for (int i = 0; i < RPT; ++i)
+        for (int k = 0; k < DC; ++k) {
+            const bool in = d0 + k < D;
+            const float *gp = gcb + (size_t)(in ? d0 + k : 0) * HW, *cp = cob + (size_t)(in ? d0 + k : 0) * HW;
 #pragma unroll
-                for (int k = 0; k < DC; ++k)
-                    tn[i][k] = (xin[i] && d0 + k < D) ? twrow[i][clampi(X - d0 - k, 0, W - 1)] : 0.f;
-        }
-#pragma unroll
-        for (int s = 0; s < NS; ++s)
-#pragma unroll
-            for (int k = 0; k < DC; ++k) {
-                const bool ok = qin[s] && d0 + k < D;
-                const size_t vo = vbase[s] + (size_t)(ok ? d0 + k : 0) * HW, so = sbase[s] - (ok ? d0 + k : 0);
-                g[s][k] = ok ? a.gc[vo] : 0.f;
-                cc[s][k] = ok ? a.cost[vo] : 1.f;
-                sb[s][k] = ok ? a.isdt[so] : 0.f;   // 1 / s_b (0: a flat target block)
-                mb[s][k] = ok ? a.mut[so] : 0.f;
+            for (int s = 0; s < NS; ++s) {
+                const bool ok = in && qin[s];
+                const int sk = so[s] - (in ? d0 + k : 0);
+                g[s][k] = ok ? gp[qo[s]] : 0.f;
+                sbv[s][k] = ok ? isb[sk] : 0.f;   // 1 / s_b (0: a flat target block)
+                if (s < NO) {
+                    cc[s][k] = ok ? cp[qo[s]] : 1.f;
+                    mb[s][k] = ok ? mub[sk] - lev.y : 0.f;
+                }
             }
+        }
     };
     load_round(0);
+    __syncthreads();   // the shared rows are zeroed
     for (int d0 = 0; d0 < D; d0 += DC) {
-        // ---- stage the window-pair terms of the halo for DC disparities
+        // ---- stage A of the halo for DC disparities; the tile's own pairs add up their sums
 #pragma unroll
         for (int s = 0; s < NS; ++s) {
             const int j = threadIdx.x + 256 * s;
             if (j >= NQ) break;
 #pragma unroll
             for (int k = 0; k < DC; ++k) {
-                float A = 0.f, C = 0.f, Bq = 0.f;
-                if (qisa[s] > 0.f && sb[s][k] > 0.f) {
-                    const float isb = sb[s][k];
-                    const float gn = g[s][k] * a.inv_n, gnc = gn * (1.f - cc[s][k]);
-                    A = -gn * qisa[s] * isb;
-                    Bq = gnc * qisa[s] * qisa[s];
-                    C = gnc * isb * isb;
+                float A = 0.f, gn = 0.f;
+                const bool live = qisa[s] > 0.f && sbv[s][k] > 0.f;
+                if (live) {
+                    gn = g[s][k] * a.inv_n;
+                    A = -gn * qisa[s] * sbv[s][k];
                 }
-                sAmb[s] = fmaf(A, mb[s][k], sAmb[s]);
-                sB[s] += Bq;
-                sBmu[s] = fmaf(Bq, qmu[s], sBmu[s]);
-                st[(0 * DC + k) * SP + qofs[s]] = A;
-                st[(1 * DC + k) * SP + qofs[s]] = A * qmu[s];
-                st[(2 * DC + k) * SP + qofs[s]] = C;
-                st[(3 * DC + k) * SP + qofs[s]] = C * mb[s][k];
+                st[k * SP + qofs[s]] = A;
+                if (s < NO) {
+                    float C = 0.f;
+                    if (live) {
+                        const float gnc = gn * (1.f - cc[s][k]);
+                        sB[s] = fmaf(gnc * qisa[s], qisa[s], sB[s]);
+                        C = gnc * sbv[s][k] * sbv[s][k];
+                    }
+                    sAmb[s] = fmaf(A, mb[s][k], sAmb[s]);
+                    if (tgt && d0 + k < D) {
+                        float2 *e = gq + (j >> 5) * GW + (j & 31) - (d0 + k) + D - 1;
+                        const float2 v = *e;
+                        *e = make_float2(fmaf(A, qmu[s], v.x), v.y + C);
+                    }
+                    __syncwarp();   // lane x at d + 1 meets the entry of lane x - 1 at d
+                }
             }
-        }
-        float tc[RPT][DC];
-        if constexpr (TPF) {
-#pragma unroll
-            for (int i = 0; i < RPT; ++i)
-#pragma unroll
-                for (int k = 0; k < DC; ++k) tc[i][k] = tn[i][k];
         }
         if (d0 + DC < D) load_round(d0 + DC);
         __syncthreads();
         // ---- box sums along rows: one running sum per (plane, halo row, half row); with the
-        // odd row strides the 32 lanes of a warp (16 rows, both halves) meet 32 distinct banks
-        for (int t = threadIdx.x; t < NP * QH * 2; t += 256) {
+        // odd row strides the lanes of a warp (16 rows, both halves) meet distinct banks
+        for (int t = threadIdx.x; t < DC * QH * 2; t += 256) {
             const int half = t & 1, pr = t >> 1;
             const int p = pr / QH, row = pr - p * QH;
-            row_box16<WN>(st + p * SP + row * SW + 16 * half, hb + p * HP + row * HW_ + 16 * half);
+            const float *in = st + p * SP + row * SW + 16 * half;
+            float *out = hb + p * HP + row * HW_ + 16 * half;
+            float v[16 + 2 * RW];
+#pragma unroll
+            for (int x = 0; x < 16 + 2 * RW; ++x) v[x] = in[x];
+            float sum = 0.f;
+#pragma unroll
+            for (int x = 0; x < WN; ++x) sum += v[x];
+            out[0] = sum;
+#pragma unroll
+            for (int x = 1; x < 16; ++x) {
+                sum += v[x + WN - 1] - v[x - 1];
+                out[x] = sum;
+            }
         }
         __syncthreads();
-        // ---- box sums along columns: one running sum per (plane, column) over the TY tile rows
-        for (int t = threadIdx.x; t < NP * 32; t += 256) {
-            const int p = t >> 5, xc = t & 31;
-            const float *col = hb + p * HP + xc;
-            float *out = vb + p * TY * 32 + xc;
-            float s = 0.f;
+        // ---- box sums along columns: one running sum per (plane, column, half of the tile rows)
+        for (int t = threadIdx.x; t < DC * 64; t += 256) {
+            constexpr int NY = TY / 2;
+            const int p = t >> 6, xc = t & 31, y0 = ((t >> 5) & 1) * NY;
+            const float *col = hb + p * HP + y0 * HW_ + xc;
+            float *out = vb + p * TY * 32 + y0 * 32 + xc;
+            float v[NY + 2 * RW];
 #pragma unroll
-            for (int i = 0; i < WN; ++i) s += col[i * HW_];
-            out[0] = s;
+            for (int y = 0; y < NY + 2 * RW; ++y) v[y] = col[y * HW_];
+            float sum = 0.f;
 #pragma unroll
-            for (int y = 1; y < TY; ++y) {
-                s += col[(y + WN - 1) * HW_] - col[(y - 1) * HW_];
-                out[y * 32] = s;
+            for (int y = 0; y < WN; ++y) sum += v[y];
+            out[0] = sum;
+#pragma unroll
+            for (int y = 1; y < NY; ++y) {
+                sum += v[y + WN - 1] - v[y - 1];
+                out[y * 32] = sum;
             }
         }
         __syncthreads();
 #pragma unroll
         for (int k = 0; k < DC; ++k) {
             const int d = d0 + k;
+            if (d < D) {
 #pragma unroll
-            for (int i = 0; i < RPT; ++i) {
-                const int o = (ty + 8 * i) * 32 + tx;
-                const float bA = vb[(0 * DC + k) * TY * 32 + o], bAm = vb[(1 * DC + k) * TY * 32 + o];
-                const float bC = vb[(2 * DC + k) * TY * 32 + o], bCm = vb[(3 * DC + k) * TY * 32 + o];
-                if (xin[i] && d < D) {
-                    const float t = TPF ? tc[i][k] : twrow[i][clampi(X - d, 0, W - 1)];
-                    if (a.gpart) gts[(ty + 8 * i) * GW + tx - d + D - 1] += fmaf(rv[i], bA, -bAm) + fmaf(t, bC, -bCm);
-                    gacc[i] = fmaf(t, bA, gacc[i]);
+                for (int i = 0; i < RPT; ++i) {
+                    const float bA = vb[k * TY * 32 + (ty + 8 * i) * 32 + tx];
+                    const int e = (ty + 8 * i) * GW + tx - d + D - 1;
+                    if (xin[i]) {
+                        if (tgt) gts[e] = fmaf(rv[i], bA, gts[e]);
+                        gacc[i] = fmaf(tr[e], bA, gacc[i]);
+                    }
                 }
             }
             __syncwarp();   // lane x at d + 1 meets the entry of lane x - 1 at d
         }
-        // the next round's staging writes st only: hb and vb are rewritten after its barrier
+        // the next round's staging writes st and gq only: hb and vb are rewritten after its barriers
     }
-    // the d-independent terms: - box(sum_d A mu_b) + r box(sum_d B) - box(sum_d B mu_a)
     __syncthreads();
-    if (a.gpart) {
-        // this tile's partial diagonal sums, one row per tile row inside the extended grid
+    if (tgt) {
+        // this tile's partial sums, one row per tile row inside the extended grid (the image)
         const int nbx = cb_tiles_x(a.Wr);
         for (int i = threadIdx.x; i < TY * GW; i += 256) {
-            const int r = i / GW, j = i - r * GW, row = blockIdx.y * TY + r;
+            const int r = i / GW, j = i - r * GW, row = blockIdx.y * TY + r, qy = Y0 - RW + r;
             if (row < a.Hr) a.gpart[(((size_t)b * a.Hr + row) * nbx + blockIdx.x) * GW + j] = gts[i];
+            if (qy >= 0 && qy < H) a.gqpart[(((size_t)b * H + qy) * nbx + blockIdx.x) * GW + j] = gq[i];
         }
     }
 #pragma unroll
-    for (int s = 0; s < NS; ++s) {
-        const int j = threadIdx.x + 256 * s;
-        if (j >= NQ) break;
-        st[0 * SP + qofs[s]] = sAmb[s];
-        st[1 * SP + qofs[s]] = sB[s];
-        st[2 * SP + qofs[s]] = sBmu[s];
+    for (int s = 0; s < NO; ++s) {
+        if (!qin[s]) continue;
+        a.samb[b * HW + qo[s]] = sAmb[s];
+        a.sb[b * HW + qo[s]] = sB[s];
     }
-    __syncthreads();
-    for (int t = threadIdx.x; t < 3 * QH; t += 256) {
-        const int p = t / QH, row = t - p * QH;
-        row_box<WN>(st + p * SP + row * SW, hb + p * HP + row * HW_);
-    }
-    __syncthreads();
 #pragma unroll
-    for (int i = 0; i < RPT; ++i) {
-        float bx[3];
-#pragma unroll
-        for (int qn = 0; qn < 3; ++qn) {
-            const float *col = hb + qn * HP + (ty + 8 * i) * HW_ + tx;
-            float sum = 0.f;
-#pragma unroll
-            for (int j = 0; j < WN; ++j) sum += col[j * HW_];
-            bx[qn] = sum;
-        }
-        const int Y = Y0 + ty + 8 * i;
-        if (xin[i])
-            a.grefx[((size_t)b * a.Hr + (Y + RW)) * a.Wr + (X + RW)] = gacc[i] - bx[0] + fmaf(rv[i], bx[1], -bx[2]);
-    }
+    for (int i = 0; i < RPT; ++i)
+        if (xin[i]) a.grefx[((size_t)b * a.Hr + (Y0 + ty + 8 * i + RW)) * a.Wr + (X + RW)] = gacc[i];
 }
 
+// The window sums of both sides, added to what the cost adjoint summed with bA:
+//   reference (SIDE 0), X in the extended grid:  gref(X) += box(p)(X) + (r(X) - level) box(sum_d B)(X),
+//     p(q) = -sum_d A mu_b - (mu_a - level) sum_d B;
+//   target (SIDE 1), Xt in [-rw-(D-1), W-1+rw] (column c = Xt + rw + D - 1):  gtw(Xt) = the tiles'
+//     partial sums of r bA + box(p)(Xt) + (t(Xt) - level) box(C')(Xt), with C'(qt) = sum_d C and
+//     p(qt) = -sum_d A mu_a - (mu_b - level) C'(qt) from the tiles' partial sums (tile bx holds the
+//     target column xe = qt + D - 1 in entry xe - 32 bx + 2 rw), added in tile order.
+// A block of 32 x 32 outputs stages the two planes with their halo and sums them along rows, then
+// along columns.  Bound by reading the partial sums (about 3 float2 per position at D = 64).
+struct BoxArgs {
+    const float *ref, *tw, *mur, *mut, *samb, *sb, *gpart;
+    const float2 *gqpart;
+    float *grefx, *gtwx;
+    int W, H, D, Wr, Hr, We, Wt, rw;
+};
+constexpr int kBoxT = 32;
 
-// Target positions Xt in [-rw-(D-1), W-1+rw] (column c = Xt + rw + D - 1): the sum over d of
-// Gamma(Xt + d, d), as the partial sums of the cost adjoint's tiles whose columns reach it
-// (tile bx holds c in entry c - 32 bx), added in tile order.
-__global__ void __launch_bounds__(256) k_dtgt_diag(const float *__restrict__ gpart, float *__restrict__ gtwx,
-                                                   int D, int Wr, int Hr, int Wt)
+template <int SIDE>
+__global__ void __launch_bounds__(256) k_dbox(const BoxArgs a)
 {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x, row = blockIdx.y, b = blockIdx.z;
-    if (c >= Wt) return;
-    const int GW = cb_diag_w(D), nbx = cb_tiles_x(Wr);
-    const int bxlo = max(0, (c - GW + 1 + 31) / 32), bxhi = min(nbx - 1, c / 32);
-    const float *p = gpart + ((size_t)b * Hr + row) * nbx * GW;
-    float s = 0.f;
-    for (int bx = bxlo; bx <= bxhi; ++bx) s += p[(size_t)bx * GW + c - 32 * bx];
-    gtwx[((size_t)b * Hr + row) * Wt + c] = s;
+    extern __shared__ float2 bx_smem[];
+    const int rw = a.rw, TW = kBoxT + 2 * rw, WN = 2 * rw + 1;
+    float2 *pl = bx_smem, *hs = pl + TW * TW;      // [TW][TW], [TW][32]
+    const int b = blockIdx.z, W = a.W, H = a.H, D = a.D;
+    const size_t HW = (size_t)H * W;
+    const int GW = cb_diag_w(D), nbx = cb_tiles_x(a.Wr);
+    const int Wp = SIDE == 0 ? W : a.We, Wo = SIDE == 0 ? a.Wr : a.Wt;   // planes' columns, outputs' columns
+    const int c0 = blockIdx.x * kBoxT, r0 = blockIdx.y * kBoxT;          // first output; planes start at - 2 rw
+    const float2 lev = cb_levels(a.ref + b * HW, a.tw + b * HW, W, H);
+    for (int i = threadIdx.x; i < TW * TW; i += 256) {
+        const int r = i / TW, c = i - r * TW, y = r0 - 2 * rw + r, x = c0 - 2 * rw + c;
+        float2 v = make_float2(0.f, 0.f);
+        if (y >= 0 && y < H && x >= 0 && x < Wp) {
+            if constexpr (SIDE == 0) {
+                const size_t o = b * HW + (size_t)y * W + x;
+                v.y = a.sb[o];
+                v.x = -a.samb[o] - (a.mur[o] - lev.x) * v.y;
+            } else {
+                const float2 *p = a.gqpart + ((size_t)b * H + y) * nbx * GW;
+                // tiles whose entry j = x - 32 bx + 2 rw lies in [0, GW)
+                const int lo = max(0, (x + 2 * rw - GW + 1 + 31) / 32), hi = min(nbx - 1, (x + 2 * rw) / 32);
+                float2 s = make_float2(0.f, 0.f);
+                for (int bx = lo; bx <= hi; ++bx) {
+                    const float2 q = p[(size_t)bx * GW + x - 32 * bx + 2 * rw];
+                    s.x += q.x;
+                    s.y += q.y;
+                }
+                v.y = s.y;
+                v.x = -s.x - (a.mut[((size_t)b * H + y) * a.We + x] - lev.y) * s.y;
+            }
+        }
+        pl[i] = v;
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < TW * kBoxT; i += 256) {
+        const int r = i / kBoxT, c = i - r * kBoxT;
+        float2 s = make_float2(0.f, 0.f);
+        for (int j = 0; j < WN; ++j) {
+            const float2 v = pl[r * TW + c + j];
+            s.x += v.x;
+            s.y += v.y;
+        }
+        hs[i] = s;
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < kBoxT * kBoxT; i += 256) {
+        const int r = i / kBoxT, c = i - r * kBoxT, row = r0 + r, col = c0 + c;
+        if (row >= a.Hr || col >= Wo) continue;
+        float2 s = make_float2(0.f, 0.f);
+        for (int j = 0; j < WN; ++j) {
+            const float2 v = hs[(r + j) * kBoxT + c];
+            s.x += v.x;
+            s.y += v.y;
+        }
+        const int yc = clampi(row - rw, 0, H - 1);
+        if constexpr (SIDE == 0) {
+            const size_t o = ((size_t)b * a.Hr + row) * a.Wr + col;
+            const float v = a.ref[b * HW + (size_t)yc * W + clampi(col - rw, 0, W - 1)] - lev.x;
+            a.grefx[o] += fmaf(v, s.y, s.x);
+        } else {
+            const int lo = max(0, (col - GW + 1 + 31) / 32), hi = min(nbx - 1, col / 32);
+            const float *p = a.gpart + ((size_t)b * a.Hr + row) * nbx * GW;
+            float g = 0.f;
+            for (int bx = lo; bx <= hi; ++bx) g += p[(size_t)bx * GW + col - 32 * bx];
+            const float v = a.tw[b * HW + (size_t)yc * W + clampi(col - rw - (D - 1), 0, W - 1)] - lev.y;
+            a.gtwx[((size_t)b * a.Hr + row) * a.Wt + col] = g + fmaf(v, s.y, s.x);
+        }
+    }
 }
 
-// The folded gradient of the warped target at column xw of row y: every extended target
-// position Xt that reads column xw after clamping (the whole left or right overhang at the
-// edges), over the rows that clamp to y.
+// Adds the overhang of every extended row (the target positions that clamp to the first or the
+// last image column) to that column's entry, one warp per row.  (Folded by the threads of the
+// edge columns, the D + rw entries were one serial chain per row and set k_dfold's time.)
+__global__ void __launch_bounds__(256) k_dfold_over(float *__restrict__ gtwx, int W, int D, int rw, int Hr, int Wt)
+{
+    const int row = blockIdx.x * 8 + (threadIdx.x >> 5), b = blockIdx.y, lane = threadIdx.x & 31;
+    if (row >= Hr) return;
+    float *g = gtwx + ((size_t)b * Hr + row) * Wt;
+    const int first = rw + D - 1;                 // entry of column 0
+    float l = 0.f, r = 0.f;
+    for (int i = lane; i < first; i += 32) l += g[i];
+    for (int i = first + W + lane; i < Wt; i += 32) r += g[i];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        l += __shfl_xor_sync(0xffffffffu, l, o);
+        r += __shfl_xor_sync(0xffffffffu, r, o);
+    }
+    if (lane == 0) {
+        g[first] += l;
+        g[first + W - 1] += r;
+    }
+}
+
+// The folded gradient of the warped target at column xw of row y: the extended target position
+// xw (the overhang added by k_dfold_over) over the rows that clamp to y.
 __device__ __forceinline__ float fold_tw(const float *__restrict__ gtwx, int b, int xw, int ylo, int yhi, int W,
                                          int D, int rw, int Hr, int Wt)
 {
-    const int tlo = xw == 0 ? -rw - (D - 1) : xw, thi = xw == W - 1 ? W - 1 + rw : xw;
     float s = 0.f;
-    for (int Y = ylo; Y <= yhi; ++Y) {
-        const float *row = gtwx + ((size_t)b * Hr + Y + rw) * Wt + rw + (D - 1);
-        for (int Xt = tlo; Xt <= thi; ++Xt) s += row[Xt];
-    }
+    for (int Y = ylo; Y <= yhi; ++Y) s += gtwx[((size_t)b * Hr + Y + rw) * Wt + rw + (D - 1) + xw];
     return s;
 }
 
-// The sum, over the warped columns xw that read source column x through clamp(xw - si),
-// of the folded warped-target gradient: the adjoint of one integer-shift gather.
+// The warped columns [lo, hi] that read source column x through clamp(xw - si) (the adjoint of
+// one integer-shift gather); empty when hi < lo.
+__device__ __forceinline__ int2 unwarp_range(int x, int si, int W)
+{
+    if (W == 1) return make_int2(0, 0);
+    if (x == 0) return make_int2(0, min(W - 1, si));
+    if (x == W - 1) return make_int2(max(0, W - 1 + si), W - 1);
+    const int xw = x + si;
+    return xw < 0 || xw > W - 1 ? make_int2(1, 0) : make_int2(xw, xw);
+}
+
+// The sum of the folded warped-target gradient over that range.  An edge column's range (a
+// run as long as the shift, times rw + 1 rows at the first and last image row) is summed by its
+// whole warp; every other column reads one entry per row.  All lanes of a warp call this with
+// x = x0 + lane.
 __device__ __forceinline__ float unwarp_sum(const float *__restrict__ gtwx, int b, int x, int si, int ylo, int yhi,
                                             int W, int D, int rw, int Hr, int Wt)
 {
-    int lo, hi;
-    if (W == 1) {
-        lo = 0;
-        hi = 0;
-    } else if (x == 0) {
-        lo = 0;
-        hi = min(W - 1, si);
-    } else if (x == W - 1) {
-        lo = max(0, W - 1 + si);
-        hi = W - 1;
-    } else {
-        lo = hi = x + si;
-        if (lo < 0 || lo > W - 1) {
-            lo = 1;
-            hi = 0;
-        }
-    }
     float s = 0.f;
-    for (int xw = lo; xw <= hi; ++xw) s += fold_tw(gtwx, b, xw, ylo, yhi, W, D, rw, Hr, Wt);
+    if (x > 0 && x < W - 1) {
+        const int2 r = unwarp_range(x, si, W);
+        if (r.x <= r.y) s = fold_tw(gtwx, b, r.x, ylo, yhi, W, D, rw, Hr, Wt);
+    }
+    const int lane = threadIdx.x & 31, x0 = x - lane;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const int e = k == 0 ? 0 : W - 1;
+        if (e < x0 || e > x0 + 31 || (k == 1 && W == 1)) continue;   // (the same on every lane)
+        const int2 r = unwarp_range(e, si, W);
+        const int n = r.y - r.x + 1;
+        float t = 0.f;
+        for (int Y = ylo; Y <= yhi; ++Y) {
+            const float *row = gtwx + ((size_t)b * Hr + Y + rw) * Wt + rw + (D - 1) + r.x;
+            for (int i = lane; i < n; i += 32) t += row[i];
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (x == e) s = t;
+    }
     return s;
 }
 
@@ -1109,10 +1225,10 @@ __global__ void __launch_bounds__(256) k_dfold(const float *__restrict__ grefx, 
                                                int D, int rw, int Wr, int Hr, int Wt, int mode)
 {
     const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y, b = blockIdx.z;
-    if (x >= W) return;
+    const bool in = x < W;
     const size_t pix = ((size_t)b * H + y) * W + x;
     const int ylo = y == 0 ? -rw : y, yhi = y == H - 1 ? H - 1 + rw : y;
-    if (gref) {
+    if (gref && in) {
         const int xlo = x == 0 ? -rw : x, xhi = x == W - 1 ? W - 1 + rw : x;
         float s = 0.f;
         for (int Y = ylo; Y <= yhi; ++Y)
@@ -1121,15 +1237,17 @@ __global__ void __launch_bounds__(256) k_dfold(const float *__restrict__ grefx, 
     }
     if (gtgt) {
         const float sv = shift[(size_t)b * H + y];
+        float g;
         if (mode == STEREO_WARP_LINEAR) {
             // tw(xw) = (1 - f) tgt(clamp(xw + k)) + f tgt(clamp(xw + k + 1))
             const LinShift ls = lin_shift(sv, W);
             const float ga = unwarp_sum(gtwx, b, x, -ls.k, ylo, yhi, W, D, rw, Hr, Wt);
             const float gb = unwarp_sum(gtwx, b, x, -ls.k - 1, ylo, yhi, W, D, rw, Hr, Wt);
-            gtgt[pix] = fmaf(ls.f, gb - ga, ga);
+            g = fmaf(ls.f, gb - ga, ga);
         } else {
-            gtgt[pix] = unwarp_sum(gtwx, b, x, row_shift(sv, W), ylo, yhi, W, D, rw, Hr, Wt);
+            g = unwarp_sum(gtwx, b, x, row_shift(sv, W), ylo, yhi, W, D, rw, Hr, Wt);
         }
+        if (in) gtgt[pix] = g;
     }
 }
 
@@ -1200,12 +1318,11 @@ cudaError_t launch_agg(const AggArgs &a, int rb, int B, cudaStream_t st)
 template <int RW>
 cudaError_t launch_cb_rw(const CbArgs &a, int B, cudaStream_t st)
 {
-    constexpr int QW = 32 + 2 * RW, QH = kCbTY + 2 * RW, NP = 4 * kCbDC;
-    const size_t smem = ((size_t)NP * ((QW | 1) * QH + 33 * QH + kCbTY * 32) + kCbTY * cb_diag_w(a.D)) * sizeof(float);
+    const size_t smem = CbShape<RW>::smem(a.D);
     cudaError_t e = cudaFuncSetAttribute(k_dcost_bwd<RW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return e;
-    dim3 grid((a.Wr + 31) / 32, (a.Hr + kCbTY - 1) / kCbTY, B);
+    dim3 grid((a.Wr + 31) / 32, (a.Hr + CbShape<RW>::TY - 1) / CbShape<RW>::TY, B);
     k_dcost_bwd<RW><<<grid, 256, smem, st>>>(a);
     return cudaGetLastError();
 }
@@ -1357,6 +1474,9 @@ extern "C" int stereo_softargmin_bwd(const stereo_diff_params *p, const float *r
     c.gc = w.gc;
     const bool need_tw = gtgt || gshift;    // the warped-target gradient feeds both
     c.gpart = need_tw ? w.gpart : nullptr;
+    c.gqpart = need_tw ? (float2 *)w.gqpart : nullptr;
+    c.samb = w.samb;
+    c.sb = w.sb;
     c.grefx = w.grefx;
     c.W = d.W;
     c.H = d.H;
@@ -1366,8 +1486,18 @@ extern "C" int stereo_softargmin_bwd(const stereo_diff_params *p, const float *r
     c.We = d.We;
     c.inv_n = 1.0f / (float)d.n;
     if ((e = launch_cb(c, d.rw, B, st)) != cudaSuccess) return cuda_error(e, who);
-    if (need_tw)
-        k_dtgt_diag<<<dim3((d.Wt + 255) / 256, d.Hr, B), 256, 0, st>>>(w.gpart, w.gtwx, d.D, d.Wr, d.Hr, d.Wt);
+    {
+        const BoxArgs x = {ref, w.tw, w.mur, w.mut, w.samb, w.sb, w.gpart, (const float2 *)w.gqpart, w.grefx, w.gtwx,
+                           d.W, d.H, d.D, d.Wr, d.Hr, d.We, d.Wt, d.rw};
+        const int TW = kBoxT + 2 * d.rw;
+        const size_t smem = (size_t)TW * (TW + kBoxT) * sizeof(float2);
+        const int nr = (d.Hr + kBoxT - 1) / kBoxT;
+        if (gref) k_dbox<0><<<dim3((d.Wr + kBoxT - 1) / kBoxT, nr, B), 256, smem, st>>>(x);
+        if (need_tw) {
+            k_dbox<1><<<dim3((d.Wt + kBoxT - 1) / kBoxT, nr, B), 256, smem, st>>>(x);
+            k_dfold_over<<<dim3((d.Hr + 7) / 8, B), 256, 0, st>>>(w.gtwx, d.W, d.D, d.rw, d.Hr, d.Wt);
+        }
+    }
     if (gref || gtgt)
         k_dfold<<<dim3((d.W + 255) / 256, d.H, B), 256, 0, st>>>(w.grefx, w.gw, w.gtwx, shift, gref, gtgt, d.W,
                                                                  d.H, d.D, d.rw, d.Wr, d.Hr, d.Wt, d.warp_mode);

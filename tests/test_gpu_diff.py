@@ -416,3 +416,21 @@ def test_energy_and_refinement_sums_at_their_edges(H, W, value):
         assert got == want or (math.isnan(got) and math.isnan(want))
     flat = sgd.refine_roll(torch.full((1, H, W), 2.5, device="cuda"), None, 0.1, 3).cpu().numpy()[0]
     assert np.allclose(flat[:, 0], 0.1) and np.allclose(flat[:, 1], 2.5, atol=1e-9) and np.allclose(flat[:, 2:], 0, atol=1e-6)
+
+
+@pytest.mark.parametrize("W,H,D,win,bil", [(31, 23, 5, 9, 3), (32, 24, 4, 9, 3), (33, 25, 6, 9, 3), (24, 16, 33, 9, 5),
+                                           (65, 49, 7, 3, 3), (56, 40, 9, 11, 5), (57, 41, 34, 13, 3), (20, 18, 70, 15, 3),
+                                           (1, 30, 5, 7, 3), (40, 1, 41, 9, 3), (97, 26, 3, 1, 3)])
+def test_gradients_at_tile_edges_match_the_oracle(W, H, D, win, bil):
+    """Sizes around the cost adjoint's 32 x 24 and 32 x 16 tiles, ranges off its four disparities a
+    round and wider than a tile, images narrower than the range; both gradients by the file's bar."""
+    rng = np.random.default_rng(W * 100 + H + D)
+    ref, tgt = rng.uniform(0, 255, (H, W)), rng.uniform(0, 255, (H, W))
+    sh = rng.uniform(-3, 6, H).astype(np.float32)
+    l, p, rts, ws = gpu_forward([ref], [tgt], [sh], D, win, bil)
+    gl = rng.normal(size=(H, W))
+    lo, gro, gto = odiff.disparity_vjp(ref, tgt, sh, D, win, bil, S0, S1, T, gl)
+    assert np.abs(l[0] - lo).max() <= L_TOL
+    gr, gt = gpu_backward(p, rts, ws, gl[None].astype(np.float32))
+    check_grad(gr[0], gro, "dS/dref", floor=1e-6)
+    check_grad(gt[0], gto, "dS/dtgt", floor=1e-6)
