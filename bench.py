@@ -35,8 +35,8 @@ SM_MAX_MHZ = 2070.0
 # in profiles/ (dram__bytes_read.sum + dram__bytes_write.sum); valid only for the kernel
 # source with this SHA-256 prefix.
 FUSED_TRAFFIC = {"sha256": "972b7216c2da1f86", "bytes": 39214848}
-FUSED_SOURCES = ("internal.cuh", "k_fused_common.cuh", "k_cost.cuh", "k_fused_tc.cuh", "k_fused_sc.cuh",
-                 "k_fused_sc.cu")
+FUSED_SOURCES = ("internal.cuh", "k_fused_common.cuh", "k_cost.cuh", "k_fused_tc.cuh", "k_sc_refine.cuh",
+                 "k_march.cuh", "k_march_128.cu", "k_refine.cuh", "k_refine.cu")
 
 
 def parse():
@@ -711,7 +711,7 @@ def run_ours(args):
     probe_s, probe_p = sg.stereo_fp32_peak_probe(2)
     roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
             "traffic": traffic,
-            "kernel": "k_fused_sc (cost + bilateral aggregation + WTA + sub-pixel: tensor-core screening with a "
+            "kernel": "k_march + k_refine (cost + bilateral aggregation + WTA + sub-pixel: tensor-core screening with a "
                       "certified bound, FP32 refinement; outputs bit for bit those of the SIMT FP32 kernel)",
             "flops_per_launch": agg_flops, "flops_per_pixel_disparity": flops_per_unit,
             "avg_launch_ms": fused_avg_ms, "launches": n_fused,
@@ -721,23 +721,23 @@ def run_ours(args):
     # the FP16 / BF16 forms do the same algorithmic work: their share of the same FP32 roofline
     for v in variants.values():
         v["fused_frac_of_fp32_roofline"] = agg_flops / (v["fused_ms"] * 1e-3) / 1e12 / peak
-    # the tensor-core forms' executed mma work: per 4 x 4 patch, chunk of 32 disparities and
-    # window row, four m16n8k16 (4096 flop each), including the zero-weight K slots (32 x 36
-    # tiles of 72 patches; bil <= 13)
+    # the tensor-core forms' executed aggregation work: per 4 x 4 patch, 32 disparities and window
+    # row, four m16n8k16 (4096 flop each), including the zero-weight K slots (strips of 32 columns,
+    # eight patches per band of four rows; bil <= 13)
     peaks = measured_peaks()
     nks = 4 + 2 * (bil // 2)
-    mma_flops = ((W + 31) // 32) * ((H + 35) // 36) * 72 * ((D + 31) // 32) * nks * 4 * 4096.0
+    mma_flops = ((W + 31) // 32) * ((H + 3) // 4) * 8 * ((D + 31) // 32) * nks * 4 * 4096.0
     for name in ("f16", "bf16"):
         t_tf = mma_flops / (variants[name]["fused_ms"] * 1e-3) / 1e12
         variants[name]["tensor_mma"] = {
             "tflops": t_tf, "peak": peaks.get("bf16_tflops"), "unit": "TFLOP/s",
             "frac": t_tf / peaks["bf16_tflops"] if peaks.get("bf16_tflops") else None,
             "peak_basis": "measured dense bf16 (same rate for fp16), MEASURED_PEAKS.json",
-            "note": "the form is bound by the cost phase and shared memory, not the tensor pipe"}
-    variants["kernel"] = {"f32": "k_fused_sc (screened FP32 form; the default)",
+            "note": "the form is bound by instruction issue (costs and weights), not the tensor pipe"}
+    variants["kernel"] = {"f32": "k_march + k_refine (screened FP32 form; the default)",
                           "f32_simt": "k_fused (the SIMT FP32 form: FP32 weights and accumulators on the CUDA cores)",
-                          "f16": "k_fused_sc, plain mode (tensor-core aggregation of the FP16 costs, FP32 accumulators)",
-                          "bf16": "k_fused_sc, plain mode (tensor-core aggregation of the BF16 costs, FP32 accumulators)"}
+                          "f16": "k_march, plain mode (tensor-core aggregation of the FP16 costs, FP32 accumulators)",
+                          "bf16": "k_march, plain mode (tensor-core aggregation of the BF16 costs, FP32 accumulators)"}
 
     line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": t_max / args.steps, "higher_is_better": True,

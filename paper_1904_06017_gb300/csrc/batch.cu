@@ -17,7 +17,19 @@ struct stereo_batch {
     std::vector<stereo_pair_desc> pairs;
     std::vector<stereo_ctx *> ctx;
     int wc = 0, dc = 0, source = 0;
-    sgb::FusedKernel kernel = nullptr;
+    sgb::FusedKernel kernel = nullptr;      // (tile code kScWC: the FP32 refinement, or null)
+    // tile code kScWC, FP32 storage: the pairs of at most 32 disparities run as k_fused_sc's tiles,
+    // the first ntile items of d_items; the others' tiles are the refinement's
+    int ntile = 0;
+    size_t tile_smem = 0;
+    // tile code kScWC: one k_march launch per instantiation the pairs need
+    struct MarchGroup {
+        sgb::MarchChoice choice;
+        int first, count;                    // its items in d_march
+    };
+    std::vector<MarchGroup> march;
+    sgb::MarchItem *d_march = nullptr;
+    int ntiles = 0;                          // (pair, tile) items of the whole batch
     size_t smem = 0;
     int nsm = 0;
     sgb::PairDesc *d_pairs = nullptr;
@@ -46,6 +58,9 @@ static void release_build(stereo_batch *b)
     cudaFree(b->d_pairs);
     cudaFree(b->d_items);
     cudaFree(b->d_counter);
+    cudaFree(b->d_march);
+    b->d_march = nullptr;
+    b->march.clear();
     b->d_pairs = nullptr;
     b->d_items = nullptr;
     b->d_counter = nullptr;
@@ -74,6 +89,64 @@ static stereo_params pair_params(const stereo_batch_params &bp, const stereo_pai
     return p;
 }
 
+// The k_march items of a batch's pairs of one chunk size: their strips in segments of at most
+// `bands` bands.
+static void march_list(const stereo_batch *b, int n, int bands, std::vector<MarchItem> &out)
+{
+    for (size_t i = 0; i < b->ctx.size(); ++i) {
+        const Geometry &g = b->ctx[i]->g;
+        if (march_n(g.rb, g.D) != n || (b->bp.cost_dtype == STEREO_F32 && g.D <= 32)) continue;
+        const int nbt = (g.H + 3) / 4, segs = (nbt + bands - 1) / bands, nb = (nbt + segs - 1) / segs;
+        for (int b0 = 0; b0 < nbt; b0 += nb)
+            for (int s = 0; s < (g.W + 31) / 32; ++s) out.push_back({(int)i, s, b0, std::min(nb, nbt - b0)});
+    }
+}
+
+// Work items and launches of tile code kScWC.  A segment costs its bands plus the lead that fills
+// its window; the items go to the SMs longest first, and the segment length is the one whose
+// total work per SM plus half an item's tail is least.
+static int build_march(stereo_batch *b)
+{
+    std::vector<MarchItem> all;
+    for (int n = 128; n >= 32; n -= 32) {
+        auto cost = [&](const MarchItem &x) {
+            const Geometry &g = b->ctx[x.pair]->g;
+            return march_chunks(g.rb, g.D) * (x.nb + march_lead(g.m) + 1);
+        };
+        std::vector<MarchItem> best;
+        double best_t = 1e30;
+        for (int bands : {256, 160, 128, 96, 80, 64, 56, 48, 40, 34, 28, 24, 20, 17, 14, 12, 10, 8, 7, 6, 5, 4, 3, 2, 1}) {
+            std::vector<MarchItem> it;
+            march_list(b, n, bands, it);
+            double total = 0, longest = 0;
+            for (const MarchItem &x : it) {
+                total += cost(x);
+                longest = std::max(longest, (double)cost(x));
+            }
+            const double t = std::max(total / (b->nsm * march_ctas(n, b->bp.cost_dtype == STEREO_F32)) + 0.5 * longest, longest);
+            if (!it.empty() && t < best_t) {
+                best_t = t;
+                best.swap(it);
+            }
+        }
+        if (best.empty()) continue;
+        std::stable_sort(best.begin(), best.end(), [&](const MarchItem &x, const MarchItem &y) { return cost(x) > cost(y); });
+        const Geometry &g = b->ctx[best[0].pair]->g;
+        const MarchChoice c = pick_march(b->bp.cost_dtype, g.rb, g.rw, g.D);
+        const int rc = cuda_error(cudaFuncSetAttribute((const void *)c.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                       (int)c.smem),
+                                  "batch: cudaFuncSetAttribute");
+        if (rc) return rc;
+        b->march.push_back({c, (int)all.size(), (int)best.size()});
+        all.insert(all.end(), best.begin(), best.end());
+    }
+    int rc = cuda_error(cudaMalloc(&b->d_march, sizeof(MarchItem) * all.size()), "batch: cudaMalloc items");
+    if (!rc)
+        rc = cuda_error(cudaMemcpy(b->d_march, all.data(), sizeof(MarchItem) * all.size(), cudaMemcpyHostToDevice),
+                        "batch: copy items");
+    return rc;
+}
+
 // Contexts, descriptors and the work list for one tile configuration.
 static int build(stereo_batch *b, int wc, int dc)
 {
@@ -91,16 +164,36 @@ static int build(stereo_batch *b, int wc, int dc)
     }
     b->wc = wc;
     b->dc = dc;
-    b->kernel = pick_fused(b->bp.cost_dtype, b->bp.bil / 2, dc, wc);
-    if (!b->kernel) {
+    const bool sc = wc == kScWC;
+    const int rb = b->bp.bil / 2;
+    b->kernel = !sc ? pick_fused(b->bp.cost_dtype, rb, dc, wc) : b->bp.cost_dtype == STEREO_F32 ? pick_refine(rb, false) : nullptr;
+    if (!fused_available(b->bp.cost_dtype, rb, dc, wc)) {
         release_build(b);
         return set_error(STEREO_ENOTSUP, "batch: no fused kernel for bil=%d dc=%d wc=%d type=%d", b->bp.bil, dc,
                          wc, b->bp.cost_dtype);
     }
     b->smem = 0;
-    for (stereo_ctx *c : b->ctx) b->smem = std::max(b->smem, c->g.smem_bytes);
-    if ((rc = cuda_error(cudaFuncSetAttribute((const void *)b->kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)b->smem),
+    b->ntile = 0;
+    b->tile_smem = 0;
+    for (stereo_ctx *c : b->ctx) {
+        const Geometry &g = c->g;
+        b->smem = std::max(b->smem, sc ? refine_smem_bytes(g) : g.smem_bytes);
+        if (sc) b->tile_smem = std::max(b->tile_smem, sc_smem_bytes(g));
+    }
+    if (b->kernel && (rc = cuda_error(cudaFuncSetAttribute((const void *)b->kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                           (int)b->smem),
+                                      "batch: cudaFuncSetAttribute"))) {
+        release_build(b);
+        return rc;
+    }
+    if (sc && (rc = build_march(b))) {
+        release_build(b);
+        return rc;
+    }
+    b->ntiles = 0;
+    if (b->kernel && sc &&
+        (rc = cuda_error(cudaFuncSetAttribute((const void *)pick_fused_sc(rb), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              (int)b->tile_smem),
                          "batch: cudaFuncSetAttribute"))) {
         release_build(b);
         return rc;
@@ -114,21 +207,28 @@ static int build(stereo_batch *b, int wc, int dc)
         const stereo_pair_desc &d = b->pairs[i];
         fill_pair_desc(b->ctx[i], d.disp_dev, d.wta_dev, d.valid_dev, hp[i]);
         const Geometry &g = b->ctx[i]->g;
+        b->ntiles += g.ntx * g.nty;
+        if (sc && b->bp.cost_dtype != STEREO_F32) continue;   // (k_march finishes the 16-bit form itself)
+        if (sc && g.D <= 32) b->ntile += g.ntx * g.nty;
         for (int ty = 0; ty < g.nty; ++ty)
             for (int tx = 0; tx < g.ntx; ++tx) items.push_back({g.Dp, i, tx | (ty << 16)});
     }
-    // heaviest tiles first (the work of a tile grows with its pair's search range)
-    std::stable_sort(items.begin(), items.end(), [](const Item &x, const Item &y) { return x.key > y.key; });
+    // heaviest tiles first (the work of a tile grows with its pair's search range), after those of
+    // k_fused_sc in tile code kScWC
+    std::stable_sort(items.begin(), items.end(), [&](const Item &x, const Item &y) {
+        const bool tx = sc && b->ctx[x.pair]->g.D <= 32, ty = sc && b->ctx[y.pair]->g.D <= 32;
+        return tx != ty ? tx : x.key > y.key;
+    });
     std::vector<int2> hi(items.size());
     for (size_t k = 0; k < items.size(); ++k) hi[k] = make_int2(items[k].pair, items[k].tile);
     b->nitems = (int)hi.size();
     if ((rc = cuda_error(cudaMalloc(&b->d_pairs, sizeof(PairDesc) * n), "batch: cudaMalloc pairs")) ||
-        (rc = cuda_error(cudaMalloc(&b->d_items, sizeof(int2) * hi.size()), "batch: cudaMalloc items")) ||
-        (rc = cuda_error(cudaMalloc(&b->d_counter, sizeof(int)), "batch: cudaMalloc counter")) ||
+        (!hi.empty() && (rc = cuda_error(cudaMalloc(&b->d_items, sizeof(int2) * hi.size()), "batch: cudaMalloc items"))) ||
+        (rc = cuda_error(cudaMalloc(&b->d_counter, 2 * sizeof(int)), "batch: cudaMalloc counter")) ||
         (rc = cuda_error(cudaMemcpy(b->d_pairs, hp.data(), sizeof(PairDesc) * n, cudaMemcpyHostToDevice),
                          "batch: copy pairs")) ||
-        (rc = cuda_error(cudaMemcpy(b->d_items, hi.data(), sizeof(int2) * hi.size(), cudaMemcpyHostToDevice),
-                         "batch: copy items"))) {
+        (!hi.empty() && (rc = cuda_error(cudaMemcpy(b->d_items, hi.data(), sizeof(int2) * hi.size(), cudaMemcpyHostToDevice),
+                         "batch: copy items")))) {
         release_build(b);
         return rc;
     }
@@ -137,12 +237,23 @@ static int build(stereo_batch *b, int wc, int dc)
 
 static int enqueue_fused(stereo_batch *b, cudaStream_t s)
 {
-    int rc = cuda_error(cudaMemsetAsync(b->d_counter, 0, sizeof(int), s), "batch: reset counter");
+    int rc = cuda_error(cudaMemsetAsync(b->d_counter, 0, 2 * sizeof(int), s), "batch: reset counter");
     if (rc) return rc;
     PairDesc unused;
     memset(&unused, 0, sizeof(unused));
-    const int grid = std::min(b->nsm, b->nitems);
-    b->kernel<<<grid, fused_threads(b->wc), b->smem, s>>>(unused, b->d_pairs, b->d_items, b->nitems, b->d_counter);
+    for (const stereo_batch::MarchGroup &m : b->march) {
+        m.choice.kernel<<<m.count, m.choice.threads, m.choice.smem, s>>>(unused, b->d_pairs, b->d_march + m.first, 0);
+        if ((rc = cuda_error(cudaGetLastError(), "batch: march launch"))) return rc;
+    }
+    if (b->ntile) {
+        pick_fused_sc(b->bp.bil / 2)<<<std::min(b->nsm, b->ntile), kThreads, b->tile_smem, s>>>(unused, b->d_pairs, b->d_items,
+                                                                                               b->ntile, b->d_counter + 1);
+        if ((rc = cuda_error(cudaGetLastError(), "batch: tile launch"))) return rc;
+    }
+    const int rest = b->nitems - b->ntile;
+    if (!rest) return STEREO_OK;            // (tile code kScWC: every pair is done)
+    const int grid = std::min(b->nsm, rest);
+    b->kernel<<<grid, fused_threads(b->wc), b->smem, s>>>(unused, b->d_pairs, b->d_items + b->ntile, rest, b->d_counter);
     return cuda_error(cudaGetLastError(), "batch: fused launch");
 }
 
@@ -219,7 +330,7 @@ static std::string tune_key(const stereo_batch *b)
 {
     std::string k;
     char buf[96];
-    snprintf(buf, sizeof(buf), "c6 w%d k%d t%d sm%d |", b->bp.win, b->bp.bil, b->bp.cost_dtype, b->nsm);
+    snprintf(buf, sizeof(buf), "c7 w%d k%d t%d sm%d |", b->bp.win, b->bp.bil, b->bp.cost_dtype, b->nsm);
     k += buf;
     for (const stereo_pair_desc &d : b->pairs) {
         snprintf(buf, sizeof(buf), " %dx%dx%d", d.width, d.height, d.max_disp);
@@ -295,7 +406,7 @@ static int autotune(stereo_batch *b, int *wc_out, int *dc_out, int *source)
 {
     const char *path = getenv("STEREO_AUTOTUNE_CACHE");
     const std::string key = tune_key(b);
-    if (cache_lookup(path, key, wc_out, dc_out) && pick_fused(b->bp.cost_dtype, b->bp.bil / 2, *dc_out, *wc_out) &&
+    if (cache_lookup(path, key, wc_out, dc_out) && fused_available(b->bp.cost_dtype, b->bp.bil / 2, *dc_out, *wc_out) &&
         (*wc_out != kTcWC || tc_supported(b->bp.cost_dtype, b->bp.bil, b->bp.sigma1))) {
         *source = 1;
         return STEREO_OK;
@@ -307,7 +418,7 @@ static int autotune(stereo_batch *b, int *wc_out, int *dc_out, int *source)
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
     for (const auto &c : cand) {
-        if (!pick_fused(b->bp.cost_dtype, b->bp.bil / 2, c[1], c[0])) continue;
+        if (!fused_available(b->bp.cost_dtype, b->bp.bil / 2, c[1], c[0])) continue;
         if (c[0] == kTcWC && !tc_supported(b->bp.cost_dtype, b->bp.bil, b->bp.sigma1)) continue;
         if (build(b, c[0], c[1]) != STEREO_OK) continue;   // e.g. shared memory does not fit
         int rc = enqueue_pre(b, b->cap);
@@ -429,7 +540,7 @@ int stereo_batch_config(const stereo_batch *b, int32_t *wc, int32_t *dc, int32_t
     if (!b || !wc || !dc || !n_items || !source) return set_error(STEREO_EINVAL, "stereo_batch_config: null pointer");
     *wc = b->wc;
     *dc = b->dc;
-    *n_items = b->nitems;
+    *n_items = b->ntiles;
     *source = b->source;
     return STEREO_OK;
 }

@@ -34,11 +34,49 @@ constexpr int kWsMaxRB = 5;         // the two cost buffers fit shared memory up
 constexpr int kTcWC = 16;
 constexpr int kTcMaxRB = 6;
 constexpr float kTcMaxSigma1 = 150.f;   // -s^2 stays a normal FP16 number
-// The screened FP32 form (tile code kScWC): 32 x 36 tiles, kWarps warps, tensor-core screening
-// over 32 disparities per chunk and an exact FP32 refinement of the certified candidates
-// (k_fused_sc.cuh); bil <= 13 (at 13 a window row fills the 16 k-slots of an mma).
+// The tensor-core form of tile code kScWC (every storage type; bil <= 13, where a window row fills
+// the 16 k-slots of an mma).  Its chunk size as a batch parameter is 32.  k_march computes and
+// aggregates 16-bit costs down strips of 32 columns; for FP32 storage the certified candidates are
+// then evaluated in FP32 on 32 x 36 tiles by k_refine.  See sc_route.
 constexpr int kScWC = 32;
 constexpr int kScMaxRB = 6;
+constexpr int kScDC = 32;
+// k_march: a band is four rows; image rows come in groups of four that start march_phi rows
+// before the segment, and a band's costs are whole march_lead groups after its first.
+__host__ __device__ constexpr int march_phi(int m) { return (m & 1) ? 2 : 0; }
+__host__ __device__ constexpr int march_lead(int m) { return (2 * m + march_phi(m)) / 4; }
+// Disparities per pass for a search range: the range in equal parts of at most 128 (96 where a
+// wider ring exceeds shared memory, bil = 13), rounded up to 32.
+__host__ __device__ constexpr int march_n(int rb, int D)
+{
+    const int most = rb <= 5 ? 128 : 96, ch = (D + most - 1) / most;
+    return ((D + ch - 1) / ch + 31) / 32 * 32;
+}
+// CTAs of k_march per SM: two in the 16-bit form with 32 disparities per chunk (80 registers a
+// thread), else one.
+__host__ __device__ constexpr int march_ctas(int n, bool f32) { return n == 32 && !f32 ? 2 : 1; }
+__host__ __device__ constexpr int march_chunks(int rb, int D)
+{
+    return (D + march_n(rb, D) - 1) / march_n(rb, D);
+}
+// How a frame of FP32 storage runs (times of stereo_cost_aggregate_wta, w = 9, k = 11 where not said):
+//   kRouteTile    k_fused_sc, screening and refinement of a 32 x 36 tile in one kernel: ranges of at
+//                 most 32, where the screening is one chunk and the refinement most of the work
+//                 (1920 x 1080, D = 32: 616 us, k_march and k_refine 629; 960 x 540: 186 against 239)
+//   kRouteMarch   k_march, then k_refine: longer ranges (1920 x 1080: D = 64 688 us against 846 by
+//                 tiles, D = 128 862 against 1372; 960 x 540, D = 64: 235 against 266; 640 x 480,
+//                 D = 64: 175 against 190; 300 x 200, D = 48, k = 7: 99 against 111)
+//   kRouteRefine  k_march with the refinement inside: ranges of at most 32 on frames of at most
+//                 kRouteSmall pixels, where the tiles are fewer than the SMs and a tile's latency is
+//                 the time (160 x 120, k = 13: 42 us against 85; 320 x 240, k = 9: 54 against 77; but
+//                 400 x 300, D = 30: 93 against 87, its refiners are slower where many candidates tie)
+enum { kRouteTile = 0, kRouteMarch = 1, kRouteRefine = 2 };
+constexpr int kRouteSmall = 81920;
+__host__ __device__ constexpr int sc_route(int W, int H, int D)
+{
+    return D > 32 ? kRouteMarch : (long long)W * H <= kRouteSmall ? kRouteRefine : kRouteTile;
+}
+constexpr int kMarchPadR = 112;     // columns k_march's staged rows may reach past a strip's first column
 __host__ __device__ constexpr int tile_x(int wc)
 {
     return wc == kWsWC || wc == kTcWC ? 64 : wc == kScWC ? 32 : 32 * wc;
@@ -82,11 +120,14 @@ struct stereo_ctx {
     stereo_params p;
     sgb::Geometry g;
     int device;
-    int nsm;                       // SMs of the device (grid of the persistent screened kernel)
+    int nsm;                       // SMs of the device
     uint8_t *ref_pad, *tgt_pad;    // replicate-padded copies (pad_pitch x pad_h)
     int2 *ref_stats, *tgt_stats;   // per padded position: {sum, bits of 1/sqrt(n*sumsq - sum^2)}
     int4 *row_tab;                 // per image row: {s_i(v), max and min of s_i over rows v-m..v+m,
                                    //   min over those rows of the target's column-0 run length}
+    int *cand;                     // [H][W] candidate ranges of the screened form (or null)
+    float *emin;                   // [H][W] running minimum between the screening's chunks (or null)
+    float *wst;                    // [6][H][W] running WTA between the 16-bit form's chunks (or null)
     CUtensorMap tmap_ref, tmap_tgt;
     float kspatial[(2 * sgb::kMaxRB + 1) * (2 * sgb::kMaxRB + 1)];  // -log2(e) |dq|^2 / sigma0^2
     float iscale;                  // sqrt(log2(e)) / sigma1
@@ -118,6 +159,8 @@ int launch_row_tables(stereo_ctx *ctx, const float *shift, const uint8_t *tgtw, 
 int launch_fused(stereo_ctx *ctx, const float *shift, float *disp, int32_t *wta, uint8_t *valid,
                  cudaStream_t s, float *best2 = nullptr);
 size_t fused_smem_bytes(const Geometry &g);
+size_t refine_smem_bytes(const Geometry &g);   // of k_refine (tile code kScWC, FP32 storage)
+size_t sc_smem_bytes(const Geometry &g);       // of k_fused_sc
 int fused_configure(stereo_ctx *ctx);
 int compute_geometry(const stereo_params &p, int dc, int wc, Geometry &g);
 // Context creation with a given (disparities per chunk, warp columns); 0 = default choice.

@@ -20,10 +20,14 @@ struct FusedArgs {
     int32_t *wta;
     uint8_t *valid;
     float *best2;       // optional [H][W][2]: normalised E at d* and the smallest E over d != d*
+    const uint8_t *ref_pad, *tgt_pad;   // the replicate-padded images the tensor maps describe
+    int *cand;          // [H][W] certified candidate range dlo | dhi << 16 (screened form)
+    float *emin;        // [H][W] running minimum between the screening's chunks
+    float *wst;         // [6][H][W] running WTA between the 16-bit form's chunks
     int *status;
     int stall_test;     // test hook: arm the staging barrier but issue no copy (the wait expires)
     int W, H, D, Dp, rw, m, n;
-    int pad_left, pad_top, pad_w;
+    int pad_left, pad_top, pad_w, pad_pitch;
     int ref_e, tgt_e, ref_box_w, tgt_box_w, box_h, ref_box_x;
     float iscale;
     float K[(2 * kMaxRB + 1) * (2 * kMaxRB + 1)];
@@ -254,16 +258,37 @@ FusedKernel pick_fused_f16(int rb, int dc, int wc);    // k_fused_f16.cu: WC = 2
 FusedKernel pick_fused_bf16(int rb, int dc, int wc);   // k_fused_bf16.cu: WC = 2, DC = 12
 FusedKernel pick_fused_ws(int rb, int dc);             // k_fused_ws.cu: warp-specialised, FP32, DC = 12
 FusedKernel pick_fused_tc(int cost_dtype, int rb);     // k_fused_tc_{f16,bf16}.cu: tensor-core aggregation, DC = 16
-FusedKernel pick_fused_sc(int rb);                     // k_fused_sc.cu: screened FP32 form, tile code kScWC
-FusedKernel pick_fused_sc_b2(int rb);                  // k_fused_sc_b2.cu: the same with the best2 output
-FusedKernel pick_fused_sc16(int cost_dtype, int rb);   // k_fused_sc16.cu: FP16 / BF16 storage, tile code kScWC
-FusedKernel pick_fused_sc16_b2(int cost_dtype, int rb);   // k_fused_sc16_b2.cu: the same with best2
+FusedKernel pick_fused_sc(int rb);                     // k_fused_sc.cu: screened FP32 tiles of tile code kScWC
+FusedKernel pick_refine(int rb, bool b2);              // k_refine.cu: FP32 refinement of tile code kScWC
 FusedKernel pick_fused(int cost_dtype, int rb, int dc, int wc);
 // The instantiation with the best2 output (FP32 storage at WC = 2 with DC = 12, and the
 // tensor-core form); nullptr where there is none.  k_fused_b2_f32.cu, k_fused_tc_{f16,bf16}_b2.cu.
 FusedKernel pick_fused_b2(int cost_dtype, int rb, int dc, int wc);
 FusedKernel pick_fused_f32_b2(int rb, int dc);
 FusedKernel pick_fused_tc_b2(int cost_dtype, int rb);
+// Whether (cost type, radius, chunk, tile code) is compiled.
+bool fused_available(int cost_dtype, int rb, int dc, int wc);
+
+// ---- k_march: one work item, bands [b0, b0 + nb) of strip `strip` of a pair
+struct MarchItem {
+    int pair, strip, b0, nb;
+};
+typedef void (*MarchKernel)(const PairDesc, const PairDesc *, const MarchItem *, int);
+// What a launch needs to know of an instantiation.
+struct MarchChoice {
+    MarchKernel kernel;
+    int threads;
+    size_t smem;
+};
+// k_march_{32,64,96,128}.cu: by disparities per chunk 
+MarchChoice pick_march_32(int cost_dtype, int rb, int rw);
+MarchChoice pick_march_64(int cost_dtype, int rb, int rw);
+MarchChoice pick_march_96(int cost_dtype, int rb, int rw);
+MarchChoice pick_march_128(int cost_dtype, int rb, int rw);
+MarchChoice pick_march(int cost_dtype, int rb, int rw, int D);   // k_march.cu
+// Bands per work item of one frame on nsm SMs, and the items of that split.
+int march_bands(int W, int H, int m, int nsm);
+int march_items(int W, int H, int bands);
 // The descriptor of one context for one call (k_fused_f32.cu).
 void fill_pair_desc(const stereo_ctx *ctx, float *disp, int32_t *wta, uint8_t *valid, PairDesc &d,
                     float *best2 = nullptr);

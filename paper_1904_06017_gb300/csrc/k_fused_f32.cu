@@ -5,7 +5,8 @@
 #include <algorithm>
 
 #include "k_fused.cuh"
-#include "k_fused_sc.cuh"
+#include "k_fused_tc.cuh"
+#include "k_refine.cuh"
 
 namespace sgb {
 
@@ -21,11 +22,7 @@ FusedKernel pick_fused(int cost_dtype, int rb, int dc, int wc)
 {
     if (wc == kWsWC) return cost_dtype == STEREO_F32 && rb <= kWsMaxRB ? pick_fused_ws(rb, dc) : nullptr;
     if (wc == kTcWC) return dc == kTcDC && rb <= kTcMaxRB ? pick_fused_tc(cost_dtype, rb) : nullptr;
-    if (wc == kScWC) {
-        if (dc != kScDC) return nullptr;
-        return cost_dtype == STEREO_F32 ? pick_fused_sc(rb) : pick_fused_sc16(cost_dtype, rb);
-    }
-    switch (cost_dtype) {
+    switch (wc == kScWC ? -1 : cost_dtype) {
     case STEREO_F32: return pick_fused_f32(rb, dc, wc);
     case STEREO_F16: return pick_fused_f16(rb, dc, wc);
     case STEREO_BF16: return pick_fused_bf16(rb, dc, wc);
@@ -33,10 +30,26 @@ FusedKernel pick_fused(int cost_dtype, int rb, int dc, int wc)
     return nullptr;
 }
 
+bool fused_available(int cost_dtype, int rb, int dc, int wc)
+{
+    if (wc == kScWC) return dc == kScDC && rb <= kScMaxRB;
+    return pick_fused(cost_dtype, rb, dc, wc) != nullptr;
+}
+
+size_t refine_smem_bytes(const Geometry &g)
+{
+    return refine_layout(g.rb, g.m, g.ref_box_w, g.tgt_box_w, g.box_h).total;
+}
+
 size_t fused_smem_bytes(const Geometry &g)
 {
     if (g.wc == kTcWC) return tc_layout(g.rb, g.m, g.ref_box_w, g.tgt_box_w, g.box_h, g.esize).total;
-    if (g.wc == kScWC) return sc_layout(g.rb, g.m, g.ref_box_w, g.tgt_box_w, g.box_h).total;
+    if (g.wc == kScWC) {
+        if (g.rb > kScMaxRB) return (size_t)1 << 30;
+        if (g.esize != 4) return pick_march(STEREO_F16, g.rb, g.rw, g.D).smem;
+        const size_t m = sc_route(g.W, g.H, g.D) == kRouteTile ? sc_smem_bytes(g) : pick_march(STEREO_F32, g.rb, g.rw, g.D).smem;
+        return std::max(m, refine_smem_bytes(g));
+    }
     // the warp-specialised form keeps the two-pass cost phase (vband, staged statistics); the
     // others compute costs on the tensor cores and need neither
     const bool ws = g.wc == kWsWC;
@@ -50,8 +63,30 @@ static FusedKernel pick(const stereo_ctx *ctx)
     return pick_fused(ctx->p.cost_dtype, ctx->g.rb, ctx->g.dc, ctx->g.wc);
 }
 
+static int set_smem(const void *k, size_t bytes, const char *what)
+{
+    return cuda_error(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes), what);
+}
+
 int fused_configure(stereo_ctx *ctx)
 {
+    const Geometry &g = ctx->g;
+    if (g.wc == kScWC) {
+        if (!fused_available(ctx->p.cost_dtype, g.rb, g.dc, g.wc))
+            return set_error(STEREO_ENOTSUP, "no tensor-core form for bil=%d dc=%d", ctx->p.bil, g.dc);
+        const bool f32 = ctx->p.cost_dtype == STEREO_F32;
+        int rc;
+        if (f32 && sc_route(g.W, g.H, g.D) == kRouteTile) {
+            rc = set_smem((const void *)pick_fused_sc(g.rb), sc_smem_bytes(g), "cudaFuncSetAttribute(tiles)");
+        } else {
+            const MarchChoice c = pick_march(ctx->p.cost_dtype, g.rb, g.rw, g.D);
+            rc = set_smem((const void *)c.kernel, c.smem, "cudaFuncSetAttribute(march)");
+        }
+        if (rc || !f32) return rc;
+        const size_t rs = refine_smem_bytes(g);
+        if ((rc = set_smem((const void *)pick_refine(g.rb, false), rs, "cudaFuncSetAttribute(refine)"))) return rc;
+        return set_smem((const void *)pick_refine(g.rb, true), rs, "cudaFuncSetAttribute(refine, best2)");
+    }
     FusedKernel k = pick(ctx);
     if (!k)
         return set_error(STEREO_ENOTSUP, "no fused kernel for bil=%d dc=%d cost_dtype=%d", ctx->p.bil, ctx->g.dc,
@@ -84,6 +119,11 @@ void fill_pair_desc(const stereo_ctx *ctx, float *disp, int32_t *wta, uint8_t *v
     a.wta = wta;
     a.valid = valid;
     a.best2 = best2;
+    a.ref_pad = ctx->ref_pad;
+    a.tgt_pad = ctx->tgt_pad;
+    a.cand = ctx->cand;
+    a.emin = ctx->emin;
+    a.wst = ctx->wst;
     a.status = ctx->status_dev;
     a.stall_test = ctx->stall_test;
     a.W = g.W;
@@ -96,6 +136,7 @@ void fill_pair_desc(const stereo_ctx *ctx, float *disp, int32_t *wta, uint8_t *v
     a.pad_left = g.pad_left;
     a.pad_top = g.pad_top;
     a.pad_w = g.pad_w;
+    a.pad_pitch = g.pad_pitch;
     a.ref_e = g.ref_e;
     a.tgt_e = g.tgt_e;
     a.ref_box_w = g.ref_box_w;
@@ -112,6 +153,27 @@ int launch_fused(stereo_ctx *ctx, const float *shift, float *disp, int32_t *wta,
 {
     (void)shift;   // the integer shifts come from the row table built by k_row_tables
     const Geometry &g = ctx->g;
+    if (g.wc == kScWC) {
+        PairDesc d;
+        fill_pair_desc(ctx, disp, wta, valid, d, best2);
+        const bool f32 = ctx->p.cost_dtype == STEREO_F32;
+        const int route = !f32 ? kRouteMarch : best2 ? kRouteTile : sc_route(g.W, g.H, g.D);
+        if (!(f32 && route == kRouteTile)) {
+            const MarchChoice c = pick_march(ctx->p.cost_dtype, g.rb, g.rw, g.D);
+            const int nb = march_bands(g.W, g.H, g.m, ctx->nsm * march_ctas(march_n(g.rb, g.D), f32));
+            c.kernel<<<march_items(g.W, g.H, nb), c.threads, c.smem, s>>>(d, nullptr, nullptr, nb);
+            const cudaError_t e = cudaGetLastError();
+            if (e != cudaSuccess || !f32 || route == kRouteRefine) return cuda_error(e, "k_march launch");
+        }
+        // persistent tiles: one CTA per SM, tiles in turn, the next tile's images staged while the
+        // current one finishes.  (With best2 every disparity is refined: nothing to screen.)
+        const int ntiles = g.ntx * g.nty;
+        const bool tile = route == kRouteTile && !best2;
+        const FusedKernel k = tile ? pick_fused_sc(g.rb) : pick_refine(g.rb, best2 != nullptr);
+        k<<<std::min(ntiles, ctx->nsm), kThreads, tile ? sc_smem_bytes(g) : refine_smem_bytes(g), s>>>(d, nullptr, nullptr, ntiles,
+                                                                                                       nullptr);
+        return cuda_error(cudaGetLastError(), "k_fused_sc / k_refine launch");
+    }
     FusedKernel k = best2 ? pick_fused_b2(ctx->p.cost_dtype, g.rb, g.dc, g.wc) : pick(ctx);
     if (!k)
         return set_error(STEREO_ENOTSUP, best2 ? "the best2 output needs FP32 storage (the screened form or 12 "
@@ -121,10 +183,7 @@ int launch_fused(stereo_ctx *ctx, const float *shift, float *disp, int32_t *wta,
     PairDesc d;
     fill_pair_desc(ctx, disp, wta, valid, d, best2);
     const int ntiles = g.ntx * g.nty;
-    // the screened form is persistent (one CTA per SM, tiles in turn, the next tile's images
-    // staged while the current one finishes); the others take one tile per CTA
-    const int grid = g.wc == kScWC ? std::min(ntiles, ctx->nsm) : ntiles;
-    k<<<grid, fused_threads(g.wc), g.smem_bytes, s>>>(d, nullptr, nullptr, ntiles, nullptr);
+    k<<<ntiles, fused_threads(g.wc), g.smem_bytes, s>>>(d, nullptr, nullptr, ntiles, nullptr);
     return cuda_error(cudaGetLastError(), "k_fused launch");
 }
 

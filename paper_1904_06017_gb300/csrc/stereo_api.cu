@@ -47,9 +47,13 @@ int compute_geometry(const stereo_params &p, int dc, int wc, Geometry &g)
     g.tx = tile_x(wc);
     g.ty = tile_y(wc);
     g.esize = p.cost_dtype == STEREO_F32 ? 4 : 2;
-    // the screened form's FP32 refinement computes 16 disparities from any start d <= D - 1,
-    // so its target strip holds 16 disparities beyond the last screening chunk
-    g.Dp = wc == kScWC ? round_up(g.D, dc) + 16 : round_up(g.D, dc);
+    // the kScWC form's FP32 refinement computes 16 disparities from any start d <= D - 1, and its
+    // passes of march_n disparities may end past D
+    g.Dp = round_up(g.D, dc);
+    if (wc == kScWC) {
+        g.Dp += 16;
+        if (g.Dp < march_chunks(g.rb, g.D) * march_n(g.rb, g.D)) g.Dp = march_chunks(g.rb, g.D) * march_n(g.rb, g.D);
+    }
     g.ntx = (g.W + g.tx - 1) / g.tx;
     g.nty = (g.H + g.ty - 1) / g.ty;
     g.pad_left = round_up(g.m + g.Dp - 1, 16);
@@ -63,6 +67,7 @@ int compute_geometry(const stereo_params &p, int dc, int wc, Geometry &g)
     int end_ref = x_last + g.pad_left - round_up(g.m, 16) + g.ref_box_w;
     int end_tgt = x_last + g.tgt_box_w;
     g.pad_w = round_up((end_ref > end_tgt ? end_ref : end_tgt), 16);
+    if (wc == kScWC && g.pad_w < x_last + g.pad_left + kMarchPadR) g.pad_w = x_last + g.pad_left + kMarchPadR;
     g.pad_h = g.nty * g.ty + 2 * g.m;
     g.pad_pitch = round_up(g.pad_w, 128);
     g.smem_bytes = fused_smem_bytes(g);
@@ -107,6 +112,9 @@ static void free_ctx(stereo_ctx *c)
     cudaFree(c->ref_stats);
     cudaFree(c->tgt_stats);
     cudaFree(c->row_tab);
+    cudaFree(c->cand);
+    cudaFree(c->emin);
+    cudaFree(c->wst);
     cudaFree(c->mom_part);
     cudaFree(c->dt_coef);
     cudaFree(c->res_dev);
@@ -244,6 +252,11 @@ int create_context(const stereo_params *p, int force_dc, int force_wc, stereo_ct
         (rc = cuda_error(cudaMalloc(&c->ref_stats, st), "cudaMalloc ref_stats")) ||
         (rc = cuda_error(cudaMalloc(&c->tgt_stats, st), "cudaMalloc tgt_stats")) ||
         (rc = cuda_error(cudaMalloc(&c->row_tab, sizeof(int4) * g.H), "cudaMalloc row table")) ||
+        (g.wc == kScWC && g.esize == 4 && g.D > 32 &&
+         (rc = cuda_error(cudaMalloc(&c->cand, sizeof(int) * g.H * g.W), "cudaMalloc candidates"))) ||
+        (g.wc == kScWC && march_chunks(g.rb, g.D) > 1 &&
+         (rc = g.esize == 4 ? cuda_error(cudaMalloc(&c->emin, sizeof(float) * g.H * g.W), "cudaMalloc minima")
+                            : cuda_error(cudaMalloc(&c->wst, 6 * sizeof(float) * g.H * g.W), "cudaMalloc WTA state"))) ||
         (rc = cuda_error(cudaMalloc(&c->mom_part, sizeof(double) * 10 * kDtMaxBlocks), "cudaMalloc moments")) ||
         (rc = cuda_error(cudaMalloc(&c->res_dev, sizeof(stereo_dt_result)), "cudaMalloc result")) ||
         (rc = cuda_error(cudaMalloc(&c->dt_coef, 4 * sizeof(float)), "cudaMalloc coefficients")) ||
