@@ -434,3 +434,56 @@ def test_gradients_at_tile_edges_match_the_oracle(W, H, D, win, bil):
     gr, gt = gpu_backward(p, rts, ws, gl[None].astype(np.float32))
     check_grad(gr[0], gro, "dS/dref", floor=1e-6)
     check_grad(gt[0], gto, "dS/dtgt", floor=1e-6)
+
+
+@pytest.mark.parametrize("W,H,D,bil", [(31, 3, 31, 11), (32, 4, 32, 11), (33, 5, 33, 11), (65, 9, 64, 9), (34, 13, 65, 13),
+                                       (70, 18, 7, 1), (40, 12, 3, 3), (45, 17, 36, 5), (64, 8, 97, 7), (37, 30, 1, 11),
+                                       (3, 40, 30, 13), (50, 21, 34, 15)])
+def test_aggregation_at_strip_and_chunk_edges_matches_the_oracle(W, H, D, bil):
+    """Sizes around the tensor-core form's 32-column strips, 4-row bands, chunks of 32 disparities in
+    groups of 4, for every window radius (15 takes the FP32 form); disparity and both gradients by the
+    file's bars, and a second backward pass on the same workspace equal to the first."""
+    rng = np.random.default_rng(W * 1000 + H * 10 + D)
+    ref, tgt = rng.uniform(0, 255, (H, W)), rng.uniform(0, 255, (H, W))
+    sh = rng.uniform(-3, 6, H).astype(np.float32)
+    l, p, rts, ws = gpu_forward([ref, ref[::-1].copy()], [tgt, tgt[::-1].copy()], [sh, sh], D, 5, bil)
+    gl = rng.normal(size=(2, H, W)).astype(np.float32)
+    gl[1] *= 1e-6                                        # each image has its own scale
+    gr, gt = gpu_backward(p, rts, ws, gl)
+    for i, (r, t) in enumerate([(ref, tgt), (ref[::-1], tgt[::-1])]):
+        lo, gro, gto = odiff.disparity_vjp(r.copy(), t.copy(), sh, D, 5, bil, S0, S1, T, gl[i].astype(np.float64))
+        assert np.abs(l[i] - lo).max() <= L_TOL
+        check_grad(gr[i], gro, "dS/dref", floor=1e-6 if i == 0 else 1e-12)
+        check_grad(gt[i], gto, "dS/dtgt", floor=1e-6 if i == 0 else 1e-12)
+    gr2, gt2 = gpu_backward(p, rts, ws, gl)
+    assert np.array_equal(gr, gr2) and np.array_equal(gt, gt2)
+
+
+@pytest.mark.parametrize("bil", [5, 11, 15])
+def test_what_is_not_finite_stays_in_its_windows(bil):
+    """A NaN in the reference image makes the disparity NaN in the bilateral windows that hold it and
+    nowhere else; a NaN in dS/dl reaches the gradients no farther than both windows and a tile of the
+    cost adjoint, whose window sums run along its 32 columns or fewer rows; and a gradient scaled by
+    2^60 or 2^-60 gives the scaled gradients (1e-6: the folds round on denormals)."""
+    W, H, D, win, rb, rw = 150, 101, 40, 5, bil // 2, 2
+    rng = np.random.default_rng(bil)
+    ref, tgt = rng.uniform(0, 255, (H, W)), rng.uniform(0, 255, (H, W))
+    sh = np.zeros(H, np.float32)
+    v, u = np.mgrid[0:H, 0:W]
+    y, x = 17, 90
+    bad = ref.copy()
+    bad[y, x] = np.nan
+    l, _, _, _ = gpu_forward([bad], [tgt], [sh], D, win, bil)
+    assert np.array_equal(np.isnan(l[0]), (abs(v - y) <= rb) & (abs(u - x) <= rb))
+    l, p, rts, ws = gpu_forward([ref], [tgt], [sh], D, win, bil)
+    gl = rng.normal(size=(1, H, W)).astype(np.float32)
+    gr, gt = gpu_backward(p, rts, ws, gl)
+    for s in (2.0 ** 60, 2.0 ** -60):
+        grs, gts = gpu_backward(p, rts, ws, gl * np.float32(s))
+        assert np.abs(grs / s - gr).max() <= 1e-6 * np.abs(gr).max()
+        assert np.abs(gts / s - gt).max() <= 1e-6 * np.abs(gt).max()
+    gl[0, y, x] = np.nan
+    gr, gt = gpu_backward(p, rts, ws, gl)
+    r = rb + rw + 32
+    assert np.isnan(gr[0, y, x]) and np.isfinite(gr[0][(abs(v - y) > r) | (abs(u - x) > r)]).all()
+    assert np.isfinite(gt[0][(abs(v - y) > r) | (u > x + r) | (u < x - r - D + 1)]).all()
