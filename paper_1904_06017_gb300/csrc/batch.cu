@@ -264,7 +264,7 @@ static int enqueue_fused(stereo_batch *b, cudaStream_t s)
     for (size_t k = 0; k < ng && !rc; ++k) {
         const stereo_batch::MarchGroup &m = b->march[k];
         m.choice.kernel<<<m.count, m.choice.threads, m.choice.smem, k ? b->side[k - 1] : s>>>(unused, b->d_pairs,
-                                                                                            b->d_march + m.first, 0);
+                                                                                            b->d_march + m.first, 0, 0, kMaxD);
         rc = cuda_error(cudaGetLastError(), "batch: march launch");
     }
     if (b->ntile && !rc) {

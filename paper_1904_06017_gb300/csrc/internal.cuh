@@ -47,9 +47,10 @@ __host__ __device__ constexpr int march_phi(int m) { return (m & 1) ? 2 : 0; }
 __host__ __device__ constexpr int march_lead(int m) { return (2 * m + march_phi(m)) / 4; }
 // Disparities per pass for a search range: the range in equal parts of at most 128 (96 where a
 // wider ring exceeds shared memory, bil = 13), rounded up to 32.
+__host__ __device__ constexpr int march_most(int rb) { return rb <= 5 ? 128 : 96; }
 __host__ __device__ constexpr int march_n(int rb, int D)
 {
-    const int most = rb <= 5 ? 128 : 96, ch = (D + most - 1) / most;
+    const int most = march_most(rb), ch = (D + most - 1) / most;
     return ((D + ch - 1) / ch + 31) / 32 * 32;
 }
 // CTAs of k_march per SM: two in the 16-bit form with 32 disparities per chunk (80 registers a
@@ -58,6 +59,15 @@ __host__ __device__ constexpr int march_ctas(int n, bool f32) { return n == 32 &
 __host__ __device__ constexpr int march_chunks(int rb, int D)
 {
     return (D + march_n(rb, D) - 1) / march_n(rb, D);
+}
+// A frame whose even split would be padded by 32 disparities or more takes two passes: chunks of
+// march_most up to here, then one of the rest, rounded to 32 (0: one pass).  The two calls of a frame,
+// even split -> two passes, FP32: 588 x 385, D = 147, w = 11, k = 9: 395 -> 376 us; 642 x 326, D = 160,
+// w = 7, k = 13: 534 -> 521; 838 x 513, D = 137, w = k = 7: 484 -> 455.
+__host__ __device__ constexpr int march_split(int rb, int D)
+{
+    const int full = (D - 1) / march_most(rb) * march_most(rb);
+    return full > 0 && full + march_n(rb, D - full) < march_chunks(rb, D) * march_n(rb, D) ? full : 0;
 }
 // How a frame of FP32 storage runs (times of stereo_cost_aggregate_wta, w = 9, k = 11 where not said):
 //   kRouteTile    k_fused_sc, screening and refinement of a 32 x 36 tile in one kernel: ranges of at

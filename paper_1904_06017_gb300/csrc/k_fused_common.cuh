@@ -273,7 +273,7 @@ bool fused_available(int cost_dtype, int rb, int dc, int wc);
 struct MarchItem {
     int pair, strip, b0, nb;
 };
-typedef void (*MarchKernel)(const PairDesc, const PairDesc *, const MarchItem *, int);
+typedef void (*MarchKernel)(const PairDesc, const PairDesc *, const MarchItem *, int, int, int);
 // What a launch needs to know of an instantiation.
 struct MarchChoice {
     MarchKernel kernel;
@@ -282,10 +282,13 @@ struct MarchChoice {
 };
 // k_march_{32,64,96,128}.cu: by disparities per chunk 
 MarchChoice pick_march_32(int cost_dtype, int rb, int rw);
+MarchChoice pick_march_32_screen(int rb, int rw);
 MarchChoice pick_march_64(int cost_dtype, int rb, int rw);
 MarchChoice pick_march_96(int cost_dtype, int rb, int rw);
 MarchChoice pick_march_128(int cost_dtype, int rb, int rw);
 MarchChoice pick_march(int cost_dtype, int rb, int rw, int D);   // k_march.cu
+// The second pass of a frame with march_split.
+MarchChoice pick_march_rest(int cost_dtype, int rb, int rw, int D);
 // Bands per work item of one frame on nsm SMs, and the items of that split.
 int march_bands(int W, int H, int m, int nsm);
 int march_items(int W, int H, int bands);

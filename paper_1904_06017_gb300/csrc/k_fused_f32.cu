@@ -81,6 +81,12 @@ int fused_configure(stereo_ctx *ctx)
         } else {
             const MarchChoice c = pick_march(ctx->p.cost_dtype, g.rb, g.rw, g.D);
             rc = set_smem((const void *)c.kernel, c.smem, "cudaFuncSetAttribute(march)");
+            if (!rc && march_split(g.rb, g.D)) {
+                const MarchChoice m = pick_march(ctx->p.cost_dtype, g.rb, g.rw, march_split(g.rb, g.D)),
+                                  r = pick_march_rest(ctx->p.cost_dtype, g.rb, g.rw, g.D);
+                rc = set_smem((const void *)m.kernel, m.smem, "cudaFuncSetAttribute(march)");
+                if (!rc) rc = set_smem((const void *)r.kernel, r.smem, "cudaFuncSetAttribute(march)");
+            }
         }
         if (rc || !f32) return rc;
         const size_t rs = refine_smem_bytes(g);
@@ -159,10 +165,16 @@ int launch_fused(stereo_ctx *ctx, const float *shift, float *disp, int32_t *wta,
         const bool f32 = ctx->p.cost_dtype == STEREO_F32;
         const int route = !f32 ? kRouteMarch : best2 ? kRouteTile : sc_route(g.W, g.H, g.D);
         if (!(f32 && route == kRouteTile)) {
-            const MarchChoice c = pick_march(ctx->p.cost_dtype, g.rb, g.rw, g.D);
-            const int nb = march_bands(g.W, g.H, g.m, ctx->nsm * march_ctas(march_n(g.rb, g.D), f32));
-            c.kernel<<<march_items(g.W, g.H, nb), c.threads, c.smem, s>>>(d, nullptr, nullptr, nb);
-            const cudaError_t e = cudaGetLastError();
+            const int split = march_split(g.rb, g.D);
+            cudaError_t e = cudaSuccess;
+            for (int lo = 0; lo < g.D && e == cudaSuccess; lo = split && !lo ? split : g.D) {
+                const int hi = split && !lo ? split : g.D;
+                const MarchChoice c = lo ? pick_march_rest(ctx->p.cost_dtype, g.rb, g.rw, g.D)
+                                         : pick_march(ctx->p.cost_dtype, g.rb, g.rw, hi);
+                const int nb = march_bands(g.W, g.H, g.m, ctx->nsm * march_ctas(march_n(g.rb, hi - lo), f32));
+                c.kernel<<<march_items(g.W, g.H, nb), c.threads, c.smem, s>>>(d, nullptr, nullptr, nb, lo, hi);
+                e = cudaGetLastError();
+            }
             if (e != cudaSuccess || !f32 || route == kRouteRefine) return cuda_error(e, "k_march launch");
         }
         // persistent tiles: one CTA per SM, tiles in turn, the next tile's images staged while the

@@ -15,6 +15,12 @@ MarchChoice pick_march(int cost_dtype, int rb, int rw, int D)
     return MarchChoice{nullptr, 0, 0};
 }
 
+MarchChoice pick_march_rest(int cost_dtype, int rb, int rw, int D)
+{
+    const int d = D - march_split(rb, D);
+    return cost_dtype == STEREO_F32 && march_n(rb, d) == 32 ? pick_march_32_screen(rb, rw) : pick_march(cost_dtype, rb, rw, d);
+}
+
 // A segment of nb bands takes nb + march_lead + 1 iterations (the lead fills the window, the last
 // band is aggregated behind the others), and
 // one CTA runs per SM: of all splits of the strips into equal segments, the one whose waves

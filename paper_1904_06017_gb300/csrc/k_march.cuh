@@ -248,7 +248,7 @@ __device__ __forceinline__ void march_eval3(const float *ring32, const float *sI
 template <int RB, int N, int MODE, typename T>
 __global__ void __launch_bounds__((MarchShape<RB, N>::threads(MODE)), march_ctas(N, MODE != kMarchPlain))
 k_march(const __grid_constant__ PairDesc single, const PairDesc *__restrict__ pairs,
-        const MarchItem *__restrict__ items, int bands_per_item)
+        const MarchItem *__restrict__ items, int bands_per_item, int dlo, int dhi)
 {
     using S = MarchShape<RB, N>;
     using X = TcOps<T>;
@@ -304,12 +304,12 @@ k_march(const __grid_constant__ PairDesc single, const PairDesc *__restrict__ pa
             const int dx = i / march_kw(RB), dy = i - dx * march_kw(RB);
             sK[i] = dy < KB ? a.K[dx * KB + dy] : 0.f;
         }
-    const int nchunks = REF ? 1 : (a.D + N - 1) / N;
+    const int nchunks = REF ? 1 : (min(a.D, dhi) - dlo + N - 1) / N;
     int gbase = 0;                                 // row groups staged by earlier chunks (barrier phases)
     __syncthreads();
 
     for (int ch = 0; ch < nchunks; ++ch, gbase += nsteps) {
-        const int d0 = ch * N;
+        const int d0 = dlo + ch * N;
         if (warp < S::PW) {
             // ------------------------------------------------------------------ producers
             const int db = warp % (N / 16), xb0 = (warp / (N / 16)) * XBW;
@@ -644,7 +644,7 @@ k_march(const __grid_constant__ PairDesc single, const PairDesc *__restrict__ pa
                         } else if constexpr (MODE == kMarchScreen) {
                             float em = inf;
                             int rg = 0;
-                            if (ch > 0 && in) {
+                            if (d0 > 0 && in) {
                                 em = a.emin[o];
                                 rg = a.cand[o];
                             }
@@ -658,7 +658,7 @@ k_march(const __grid_constant__ PairDesc single, const PairDesc *__restrict__ pa
                             __syncwarp();                          // the quad has read the earlier state
                             if (t4 == 0 && in) {
                                 a.cand[o] = rg;
-                                if (ch + 1 < nchunks) a.emin[o] = nm;
+                                if (d0 + N < a.D) a.emin[o] = nm;
                             }
                         } else {
                             // k_fused's running WTA over the chunks: {best, E(d* - 1), E(d* + 1), last value}
@@ -666,7 +666,7 @@ k_march(const __grid_constant__ PairDesc single, const PairDesc *__restrict__ pa
                             int bd = -1;
                             const bool b2 = a.best2 != nullptr;
                             const size_t HWs = (size_t)a.W * a.H;
-                            if (ch > 0 && in) {
+                            if (d0 > 0 && in) {
                                 best = a.wst[o];
                                 bm1 = a.wst[HWs + o];
                                 bp1 = a.wst[2 * HWs + o];
@@ -701,7 +701,7 @@ k_march(const __grid_constant__ PairDesc single, const PairDesc *__restrict__ pa
                             }
                             __syncwarp();                          // the quad has read the earlier state
                             if (t4 == 0 && in) {
-                                if (ch + 1 < nchunks) {
+                                if (d0 + N < a.D) {
                                     a.wst[o] = best;
                                     a.wst[HWs + o] = bm1;
                                     a.wst[2 * HWs + o] = bp1;

@@ -10,4 +10,7 @@ MarchChoice pick_march_32(int cost_dtype, int rb, int rw)
     return pick_march_rb<32, kMarchPlain, __nv_bfloat16>(rb, rw);
 }
 
+// Screening alone: the second pass of a longer range (march_split).
+MarchChoice pick_march_32_screen(int rb, int rw) { return pick_march_rb<32, kMarchScreen, __half>(rb, rw); }
+
 }  // namespace sgb

@@ -77,3 +77,13 @@ def test_16_bit_forms_over_chunks(dtype, gap, W, H, D, win, bil):
     b = b2.cpu().numpy()
     assert np.abs(b[..., 0] - eb).max() <= gap / 2 and np.abs(b[..., 1] - es)[sure].max() <= gap / 2
     assert np.array_equal(valid.cpu().numpy(), oracle.valid_mask(W, H, D, win, bil, shift))
+
+
+@pytest.mark.parametrize("W,H,D,bil", [(70, 21, 160, 11), (70, 21, 161, 11), (40, 30, 224, 7), (65, 17, 225, 9),
+                                       (50, 26, 160, 13), (50, 26, 161, 13), (97, 13, 224, 13), (97, 13, 225, 13)])
+def test_fp32_range_in_two_passes_equals_simt(W, H, D, bil):
+    """On both sides of the ranges whose last chunk is a pass of its own."""
+    ref, tgt, _ = pair(W, H, 5, W * 7 + H + D)
+    shift = (np.arange(H) % 5 - 2).astype(np.float32)
+    assert_same(run(ref, tgt, shift, D, 7, bil, 3.0, 10.0, sg.STEREO_FUSED_SIMT),
+                run(ref, tgt, shift, D, 7, bil, 3.0, 10.0, sg.STEREO_FUSED_TENSOR))
