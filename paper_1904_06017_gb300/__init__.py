@@ -174,6 +174,8 @@ def _ptr(x):
 def _stream(stream):
     if stream is None:
         import torch
+        if torch.cuda.is_initialized():       # the handle alone: no Stream object is made for each call
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
         return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, int):
         return stream

@@ -68,16 +68,23 @@ __global__ void __launch_bounds__(256) k_fit_partials(const float *__restrict__ 
     }
 }
 
-// Thread 0 adds the partials in block order and solves the 2 x 2 normal equations; then the
-// block writes s(v) = c0 + c1 v - delta_p.
+// Five lanes add the partials, each one sum in block order, and thread 0 solves the 2 x 2 normal
+// equations; then the block writes s(v) = c0 + c1 v - delta_p.  Bound by the chain of 64 FP64 additions
+// and the divisions; the loads are issued together (one thread walking all 320: 16 us).
 __global__ void __launch_bounds__(256) k_fit_finish(const double *__restrict__ part, int F, double delta_p,
                                                     double *__restrict__ coef, float *__restrict__ shift, int H)
 {
-    __shared__ double c[2];
+    __shared__ double c[2], sp[kFitBlocks * 5], S[5];
+    for (int i = threadIdx.x; i < kFitBlocks * 5; i += blockDim.x) sp[i] = part[i];
+    __syncthreads();
+    if (threadIdx.x < 5) {
+        double sum = 0.0;
+#pragma unroll 16
+        for (int j = 0; j < kFitBlocks; ++j) sum += sp[j * 5 + threadIdx.x];
+        S[threadIdx.x] = sum;
+    }
+    __syncthreads();
     if (threadIdx.x == 0) {
-        double S[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-        for (int j = 0; j < kFitBlocks; ++j)
-            for (int k = 0; k < 5; ++k) S[k] += part[j * 5 + k];
         const double det = S[0] * S[2] - S[1] * S[1];
         double c0 = nan(""), c1 = nan("");
         if (S[0] >= 2.0 && det > 0.0) {
