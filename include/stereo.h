@@ -79,7 +79,7 @@ typedef struct {
  *                        tensor cores with a certified error bound, the certified candidates
  *                        refined with the SIMT form's FP32 arithmetic; its outputs equal the SIMT
  *                        form's bit for bit (bil <= 13).  FP16 / BF16 storage: the tensor-core
- *                        aggregation of the 16-bit costs on the screened form's 32 x 36 tiles,
+ *                        aggregation of the 16-bit costs down strips of 32 columns,
  *                        with weights rounded from the FP32 ones (bil <= 13).  (Batches may also
  *                        take 64 x 36 tiles with weights formed in 16-bit arithmetic, tile_wc 16.)
  *   STEREO_FUSED_AUTO    TENSOR where it applies, else SIMT.
@@ -236,9 +236,10 @@ typedef struct {
                                   warps while consumer warps aggregate (FP32 storage, tile_dc 12,
                                   bil <= 11); 16: 64x36 tiles with the aggregation on the tensor cores
                                   (FP16 / BF16 storage, tile_dc 16, bil <= 13, sigma1 <= 150);
-                                  32: 32x36 tiles with the aggregation on the tensor cores, 32
-                                  disparities per chunk (tile_dc 32, bil <= 13; FP32 storage: the
-                                  screened form, see stereo_params.fused_form); 0 = autotune */
+                                  32: strips of 32 columns with the aggregation on the tensor cores
+                                  (tile_dc 32, bil <= 13; FP32 storage: the screened form, with 32x36
+                                  tiles for the refinement and for ranges of at most 32, see
+                                  stereo_params.fused_form); 0 = autotune */
     int32_t tile_dc;           /* disparities per chunk (12 or 4; 16 with tile_wc 16; 32 with
                                   tile_wc 32); 0 = autotune */
 } stereo_batch_params;

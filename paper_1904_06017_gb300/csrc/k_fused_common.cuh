@@ -259,7 +259,8 @@ FusedKernel pick_fused_bf16(int rb, int dc, int wc);   // k_fused_bf16.cu: WC = 
 FusedKernel pick_fused_ws(int rb, int dc);             // k_fused_ws.cu: warp-specialised, FP32, DC = 12
 FusedKernel pick_fused_tc(int cost_dtype, int rb);     // k_fused_tc_{f16,bf16}.cu: tensor-core aggregation, DC = 16
 FusedKernel pick_fused_sc(int rb);                     // k_fused_sc.cu: screened FP32 tiles of tile code kScWC
-FusedKernel pick_refine(int rb, bool b2);              // k_refine.cu: FP32 refinement of tile code kScWC
+// k_refine.cu: FP32 refinement of tile code kScWC, tiles of 36 rows or (without best2) kRefineRows
+FusedKernel pick_refine(int rb, bool b2, int rows = tile_y(kScWC), int ctas = 1);
 FusedKernel pick_fused(int cost_dtype, int rb, int dc, int wc);
 // The instantiation with the best2 output (FP32 storage at WC = 2 with DC = 12, and the
 // tensor-core form); nullptr where there is none.  k_fused_b2_f32.cu, k_fused_tc_{f16,bf16}_b2.cu.

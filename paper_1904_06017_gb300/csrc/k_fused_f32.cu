@@ -36,9 +36,9 @@ bool fused_available(int cost_dtype, int rb, int dc, int wc)
     return pick_fused(cost_dtype, rb, dc, wc) != nullptr;
 }
 
-size_t refine_smem_bytes(const Geometry &g)
+size_t refine_smem_bytes(const Geometry &g, int rows)
 {
-    return refine_layout(g.rb, g.m, g.ref_box_w, g.tgt_box_w, g.box_h).total;
+    return refine_layout(g.rb, g.m, g.ref_box_w, g.tgt_box_w, g.box_h, rows).total;
 }
 
 size_t fused_smem_bytes(const Geometry &g)
@@ -90,6 +90,10 @@ int fused_configure(stereo_ctx *ctx)
         }
         if (rc || !f32) return rc;
         const size_t rs = refine_smem_bytes(g);
+        for (int ctas = 1; ctas <= 2; ++ctas)
+            if ((rc = set_smem((const void *)pick_refine(g.rb, false, kRefineRows, ctas), refine_smem_bytes(g, kRefineRows),
+                               "cudaFuncSetAttribute(refine)")))
+                return rc;
         if ((rc = set_smem((const void *)pick_refine(g.rb, false), rs, "cudaFuncSetAttribute(refine)"))) return rc;
         return set_smem((const void *)pick_refine(g.rb, true), rs, "cudaFuncSetAttribute(refine, best2)");
     }
@@ -177,13 +181,16 @@ int launch_fused(stereo_ctx *ctx, const float *shift, float *disp, int32_t *wta,
             }
             if (e != cudaSuccess || !f32 || route == kRouteRefine) return cuda_error(e, "k_march launch");
         }
-        // persistent tiles: one CTA per SM, tiles in turn, the next tile's images staged while the
-        // current one finishes.  (With best2 every disparity is refined: nothing to screen.)
-        const int ntiles = g.ntx * g.nty;
+        // persistent tiles: one CTA per SM (two of k_refine's low tiles), tiles in turn, the next tile's
+        // images staged while the current one finishes.  (With best2 every disparity is refined: nothing
+        // to screen.)
         const bool tile = route == kRouteTile && !best2;
-        const FusedKernel k = tile ? pick_fused_sc(g.rb) : pick_refine(g.rb, best2 != nullptr);
-        k<<<std::min(ntiles, ctx->nsm), kThreads, tile ? sc_smem_bytes(g) : refine_smem_bytes(g), s>>>(d, nullptr, nullptr, ntiles,
-                                                                                                       nullptr);
+        const int rows = tile || best2 ? g.ty : refine_rows(g.ntx * g.nty, ctx->nsm);
+        const int ntiles = g.ntx * ((g.H + rows - 1) / rows);
+        const int ctas = tile || best2 ? 1 : refine_ctas(g.ntx * g.nty, ctx->nsm, g.rb);
+        const FusedKernel k = tile ? pick_fused_sc(g.rb) : pick_refine(g.rb, best2 != nullptr, rows, ctas);
+        k<<<std::min(ntiles, ctas * ctx->nsm), kThreads, tile ? sc_smem_bytes(g) : refine_smem_bytes(g, rows), s>>>(d, nullptr, nullptr,
+                                                                                                       ntiles, nullptr);
         return cuda_error(cudaGetLastError(), "k_fused_sc / k_refine launch");
     }
     FusedKernel k = best2 ? pick_fused_b2(ctx->p.cost_dtype, g.rb, g.dc, g.wc) : pick(ctx);

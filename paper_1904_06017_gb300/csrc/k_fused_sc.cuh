@@ -366,7 +366,7 @@ k_fused_sc(const __grid_constant__ PairDesc single, const PairDesc *__restrict__
         }
         int2 *rstr = reinterpret_cast<int2 *>(cb32 + (size_t)DCR * PSZ);   // [kScRBand4][QW]
         int2 *rstt = rstr + kScRBand4 * QW;                                  // [kScRBand4][QW + DCR - 1]
-        sc_refine<RB, false, kThreads, DCR, kScRSeg>(a, sref, stgt, cb32, vband, rstr, rstt, sIr, sKr, x0, y0, tid, &s_rlo, &s_rhi,
+        sc_refine<RB, false, kThreads, DCR, kScRSeg, TY>(a, sref, stgt, cb32, vband, rstr, rstt, sIr, sKr, x0, y0, tid, &s_rlo, &s_rhi,
                                          [&](int py, int px) {
                                              const int r = __float_as_int(sst[py * TX + px].y);
                                              return make_int2(r & 0xffff, r >> 16);

@@ -5,6 +5,11 @@
 
 namespace sgb {
 
-FusedKernel pick_refine(int rb, bool b2) { return b2 ? pick_refine_rb<true>(rb) : pick_refine_rb<false>(rb); }
+FusedKernel pick_refine(int rb, bool b2, int rows, int ctas)
+{
+    if (rows == kRefineRows)
+        return ctas == 2 ? pick_refine_rb<false, kRefineRows, 2>(rb) : pick_refine_rb<false, kRefineRows, 1>(rb);
+    return b2 ? pick_refine_rb<true, tile_y(kScWC), 1>(rb) : pick_refine_rb<false, tile_y(kScWC), 1>(rb);
+}
 
 }  // namespace sgb

@@ -2,7 +2,8 @@
 // candidate ranges that k_march certified (k_march.cuh states the bound), so that the step's
 // outputs are bit for bit those of k_fused, the plain FP32 kernel.
 //
-// A persistent CTA takes 32 x 36 tiles in turn.  Per tile it refines [dlo - 1, dhi + 1] of every
+// A persistent CTA takes tiles of 32 columns and TY rows in turn (36, or kRefineRows with one or two CTAs
+// per SM: refine_rows states where the line lies and what both sides measured).  Per tile it refines [dlo - 1, dhi + 1] of every
 // pixel (sc_refine): FP32 costs of the tile's candidate disparities from the two-pass cost phase
 // (the same integers and roundings as k_fused's), the weight ex2(fma(-t, t, K)), and the FMA
 // chain in k_fused's order (window column outer, row inner), then k_fused's running WTA in
@@ -26,10 +27,10 @@ struct RefineLayout {
     size_t sref, stgt, cbuf, vband, sstr, sstt, sI, sK, total;
 };
 
-__host__ __device__ inline RefineLayout refine_layout(int rb, int m, int ref_box_w, int tgt_box_w, int box_h)
+__host__ __device__ inline RefineLayout refine_layout(int rb, int m, int ref_box_w, int tgt_box_w, int box_h, int TY)
 {
     RefineLayout L;
-    const int TX = tile_x(kScWC), TY = tile_y(kScWC);
+    const int TX = tile_x(kScWC);
     const int QH = TY + 2 * rb, QW = TX + 2 * rb, CW = TX + 2 * m;
     const size_t v8 = (size_t)kScRBand8 * CW * 8 * 4, v4 = (size_t)kScRBand4 * CW * 4 * 4;
     L.sref = 0;
@@ -44,12 +45,12 @@ __host__ __device__ inline RefineLayout refine_layout(int rb, int m, int ref_box
     return L;
 }
 
-template <int RB, bool B2>
-__global__ void __launch_bounds__(kThreads, 1)
+template <int RB, bool B2, int TY, int CTAS>
+__global__ void __launch_bounds__(kThreads, CTAS)
 k_refine(const __grid_constant__ PairDesc single, const PairDesc *__restrict__ pairs, const int2 *__restrict__ items,
          int nitems, int *__restrict__ counter)
 {
-    constexpr int TX = tile_x(kScWC), TY = tile_y(kScWC);
+    constexpr int TX = tile_x(kScWC);
     constexpr int KB = 2 * RB + 1;
     constexpr int QH = TY + 2 * RB, QW = TX + 2 * RB;
     static_assert(RB <= kScMaxRB && QW <= kScRPW, "a row of cost positions fits the planes' pitch");
@@ -87,7 +88,7 @@ k_refine(const __grid_constant__ PairDesc single, const PairDesc *__restrict__ p
         }
         __syncthreads();
         const int RP = a.ref_box_w;
-        const RefineLayout L = refine_layout(RB, a.m, RP, a.tgt_box_w, a.box_h);
+        const RefineLayout L = refine_layout(RB, a.m, RP, a.tgt_box_w, a.box_h, TY);
         uint8_t *sref = smem + L.sref;
         uint8_t *stgt = smem + L.stgt;
         float *sIr = reinterpret_cast<float *>(smem + L.sI), *sKr = reinterpret_cast<float *>(smem + L.sK);
@@ -117,7 +118,7 @@ k_refine(const __grid_constant__ PairDesc single, const PairDesc *__restrict__ p
             const int dx = i / sc_krw(RB), dy = i - dx * sc_krw(RB);
             sKr[i] = dy < KB ? a.K[dx * KB + dy] : 0.f;
         }
-        sc_refine<RB, B2, kThreads, kScDCR, kScRSeg>(
+        sc_refine<RB, B2, kThreads, kScDCR, kScRSeg, TY>(
             a, sref, stgt, reinterpret_cast<float *>(smem + L.cbuf), reinterpret_cast<int *>(smem + L.vband),
             reinterpret_cast<int2 *>(smem + L.sstr), reinterpret_cast<int2 *>(smem + L.sstt), sIr, sKr, x0, y0, tid, &s_rlo,
             &s_rhi,
@@ -131,17 +132,17 @@ k_refine(const __grid_constant__ PairDesc single, const PairDesc *__restrict__ p
     }
 }
 
-template <bool B2>
+template <bool B2, int TY, int CTAS>
 FusedKernel pick_refine_rb(int rb)
 {
     switch (rb) {
-    case 0: return k_refine<0, B2>;
-    case 1: return k_refine<1, B2>;
-    case 2: return k_refine<2, B2>;
-    case 3: return k_refine<3, B2>;
-    case 4: return k_refine<4, B2>;
-    case 5: return k_refine<5, B2>;
-    case 6: return k_refine<6, B2>;
+    case 0: return k_refine<0, B2, TY, CTAS>;
+    case 1: return k_refine<1, B2, TY, CTAS>;
+    case 2: return k_refine<2, B2, TY, CTAS>;
+    case 3: return k_refine<3, B2, TY, CTAS>;
+    case 4: return k_refine<4, B2, TY, CTAS>;
+    case 5: return k_refine<5, B2, TY, CTAS>;
+    case 6: return k_refine<6, B2, TY, CTAS>;
     }
     return nullptr;
 }

@@ -1,4 +1,4 @@
-// k_sc_refine.cuh -- k_fused's FP32 arithmetic over the certified candidate ranges of one 32 x 36
+// k_sc_refine.cuh -- k_fused's FP32 arithmetic over the certified candidate ranges of one 32 x TY
 // tile (sc_refine), and the persistent tiles' claiming and staging: shared by k_fused_sc (screening
 // and refinement in one kernel) and k_refine (behind k_march).
 #pragma once
@@ -53,13 +53,13 @@ __device__ __forceinline__ float sc_thr(float m) { return fmaf(m + kScAbs, kScRh
 // synchronises before it reads sIr and returns after the epilogue, without a final barrier.
 // images_free() is called by every thread right after the barrier that ends the last chunk's
 // cost phase: sref and stgt are not read after it.
-template <int RB, bool B2, int NT, int DCR, int RKSEG, typename RangeOf, typename OnFree>
+template <int RB, bool B2, int NT, int DCR, int RKSEG, int TY, typename RangeOf, typename OnFree>
 __device__ __forceinline__ void sc_refine(const FusedArgs &a, const uint8_t *sref, const uint8_t *stgt, float *cb32,
                                           int *vband, int2 *sstr, int2 *sstt, const float *sIr, const float *sKr,
                                           int x0, int y0, int tid, int *s_rlo, int *s_rhi, RangeOf range_of,
                                           OnFree images_free)
 {
-    constexpr int TX = tile_x(kScWC), TY = tile_y(kScWC);
+    constexpr int TX = tile_x(kScWC);
     constexpr int KB = 2 * RB + 1, QH = TY + 2 * RB;
     constexpr int RPW = kScRPW, PSZ = sc_psz(QH);
     constexpr int NW = NT / 32, RPY = TY / NW;

@@ -87,3 +87,15 @@ def test_fp32_range_in_two_passes_equals_simt(W, H, D, bil):
     shift = (np.arange(H) % 5 - 2).astype(np.float32)
     assert_same(run(ref, tgt, shift, D, 7, bil, 3.0, 10.0, sg.STEREO_FUSED_SIMT),
                 run(ref, tgt, shift, D, 7, bil, 3.0, 10.0, sg.STEREO_FUSED_TENSOR))
+
+
+@pytest.mark.parametrize("W,H,D,win,bil", [(40, 11, 40, 9, 11), (33, 12, 40, 9, 11), (64, 13, 64, 5, 9), (70, 24, 36, 11, 7),
+                                           (33, 25, 50, 9, 13), (96, 37, 40, 3, 5), (300, 120, 140, 9, 11),
+                                           (960, 540, 40, 9, 11), (960, 541, 40, 9, 11)])
+def test_refinement_tile_heights_equal_simt(W, H, D, win, bil):
+    """Frames around the low refinement tiles' 12 rows, and on both sides of the size where the tiles
+    have 36 rows (960 x 541 has 480 of them)."""
+    ref, tgt, _ = pair(W, H, 5, W * 3 + H + D)
+    shift = (np.arange(H) % 5 - 2).astype(np.float32)
+    assert_same(run(ref, tgt, shift, D, win, bil, 3.0, 10.0, sg.STEREO_FUSED_SIMT),
+                run(ref, tgt, shift, D, win, bil, 3.0, 10.0, sg.STEREO_FUSED_TENSOR))
