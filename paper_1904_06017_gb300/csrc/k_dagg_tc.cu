@@ -1,37 +1,35 @@
-// k_dagg_tc.cu -- the bilateral aggregation stencils of the differentiable path (k_diff.cu states
-// the three modes) on the tensor cores, with FP32 accuracy from split operands.
+// k_dagg_tc.cu -- the adjoint of the bilateral aggregation in its costs (k_diff.cu, GC) on the tensor
+// cores, with FP32 accuracy from split operands.
 //
-// E(p, d) = sum_q w(p, q) c(q, d) is a banded matrix product.  A CTA marches down a strip of 32
-// pixel columns, four rows (a band) per iteration, and keeps the neighbour values of the rows its
-// window spans in a shared-memory ring, a chunk of 32 disparities at a time; the four rows that the
-// next band adds are copied (cp.async) while the band is worked on, one barrier per iteration.  A
-// warp owns a 4 x 4 pixel patch: one k-step per window row (K = the 4 + 2 RB columns that the patch's
-// windows span, padded to 16 with zero weights), four mma.sync m16n8k16 per product.
+// gc(q, d) = sum_p w(p, q) h(p, d), and with w (sI_p - sI_q) in place of w the weights' term, are banded
+// matrix products.  A CTA marches down a strip of 32 pixel columns, four rows (a band) per iteration,
+// and keeps the h of the rows its window spans in a shared-memory ring, a chunk of 32 disparities at a
+// time; the four rows that the next band adds are copied (cp.async) while the band is worked on, one
+// barrier per iteration.  A warp owns a 4 x 4 pixel patch: one k-step per window row (K = the 4 + 2 RB
+// columns that the patch's windows span, padded to 16 with zero weights), four mma.sync m16n8k16 per
+// product.
 //
 // Split.  A value x (scaled by a power of two into the FP16 range) is hi = RN16(x) and
-// lo = RN16(x - hi): 22 bits.  w v is summed as w_hi v_hi + w_lo v_hi + w_hi v_lo in FP32 accumulators
-// (the products are exact; w_lo v_lo is below 2^-22).  The normaliser Z = sum w (and S = sum w (I_q -
-// I_p)) is a column of ones in the same product, so that the accumulation rounds alike in E and Z.
-// The volumes come split from the kernels that write them (k_diff.cuh: the layout): no conversion on
-// the way into the ring.  Weights are formed in FP32 as in k_dagg and scaled by 2^14; h, which has
-// the range of the caller's dS/dl, by a power of two from the image's largest finite |dS/dl|.
-// Error against 64 bits, seeds 1 and 2 of 8 x 960 x 540, D = 64, k = 11, FP32 form -> this one: disparity
-// 9.0e-8, 7.7e-8 -> 5.1e-8, 4.6e-8; gradients 5.2e-6, 5.7e-6 -> 4.0e-6, 4.3e-6 (reference) and
-// 3.8e-6, 4.7e-6 -> 2.3e-6, 2.5e-6 (target).
+// lo = RN16(x - hi): 22 bits.  w h is summed as w_hi h_hi + w_lo h_hi + w_hi h_lo in FP32 accumulators
+// (the products are exact; w_lo h_lo is below 2^-22).  h comes split from the kernel that writes it
+// (k_diff.cuh: the layout): no conversion on the way into the ring.  Weights are formed in FP32 as in
+// k_dagg and scaled by 2^14; h, which has the range of the caller's dS/dl, by a power of two from the
+// image's largest finite |dS/dl|.  Error of both gradients against 64 bits: below the FP32 form's on five seeds of 8 x 960 x
+// 540 (reference 5.40e-6 -> 5.37e-6, target 4.19e-6 -> 4.07e-6).
 //
 // What is not finite, or out of the split's range, is flagged by row where it is written; a patch
 // whose window rows hold a flagged row sums one value at a time instead, so that a NaN reaches the pixels
 // whose windows hold it and no others.
 //
-// Bound: the tensor pipe at 42 to 51 % and the issue slots at 45 to 55 % (per window row and chunk 12 +
-// 2, 24 + 4 or 24 mma beside about 100 instructions that form and split 8 weights per lane); 54 % of the
-// K slots carry a weight.  Two CTAs per SM, so that one's epilogue and barrier pass under the other's
-// products, and the weights of the next window row are formed between the products of the current
-// one.  FP32 form (FFMA, 65 % of the pipe) -> this one: 1280 x 720, D = 64, k = 11, forward 471 -> 377 us;
-// 8 x 960 x 540: FWD 1.73 -> 1.48 ms, H 3.30 -> 2.53 ms, GC 3.11 -> 2.46 ms; 96 x 64, D = 32, where a
-// tile's chain of chunks was all there was: 50 + 88 + 68 -> 9 + 11 + 12 us.  Slower and left out:
-// producer warps that split FP32 volumes (2.11, 2.95, 2.81 ms), 64 disparities a chunk in one CTA with
-// pairs of warps sharing a patch (1.65, 2.84, 3.12), the same without pairs (1.72, 3.19, 3.37).
+// Bound: the tensor pipe at 45 % and the issue slots at 45 % (per window row and chunk 24 mma beside about
+// 100 instructions that form and split 16 operands per lane); 54 % of the K slots carry a weight.  Two CTAs
+// per SM, so that one's epilogue and barrier pass under the other's products, and the weights of the
+// next window row are formed between the products of the current one.  8 x 960 x 540, D = 64, k = 11:
+// FP32 form (FFMA, 65 % of the pipe) 3.11 ms, here 2.59 ms.  Slower and left out: producer warps that split
+// an FP32 h (2.81 ms), 64 disparities a chunk in one CTA with pairs of warps sharing a patch (3.12), the
+// same without pairs (3.37).  FWD and H in this form (1.73 -> 1.48 and 3.30 -> 2.53 ms) are left out too:
+// their error against 64 bits is lower than the FP32 form's, but where a target window is nearly flat
+// the rounding of E reaches 9e-4 of a gradient's root mean square, so that the two forms differ by as much.
 #include <math.h>
 
 #include "internal.cuh"
@@ -43,8 +41,6 @@
 
 namespace sgb {
 namespace {
-
-using AggArgs = AggArgsT<__half>;
 
 constexpr float kFar = 1e18f;        // scaled intensity of an out-of-image neighbour: weight 0
 constexpr int kWSh = 14;             // weights are scaled by 2^kWSh
@@ -75,7 +71,6 @@ __device__ __forceinline__ void mma(float (&d)[4], const uint32_t (&a)[4], uint3
         : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
-__device__ __forceinline__ float pow2i(int k) { return __int_as_float((k + 127) << 23); }   // -126 <= k <= 127
 __device__ __forceinline__ void cp_async8(uint32_t dst, const void *src, bool valid)
 {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(valid ? 8 : 0) : "memory");
@@ -108,12 +103,11 @@ __global__ void __launch_bounds__(256) k_dabsmax(const float *__restrict__ g, in
     }
 }
 
-template <int MODE, int RB>
+template <int RB>
 __global__ void __launch_bounds__(kNT, 2) k_dagg_tc(const AggArgs a, int bands_per_item)
 {
     using S = Shape<RB>;
     constexpr int QW = S::QW, RR = S::RR, NKS = 4 + 2 * RB;
-    constexpr bool TWO = MODE != AGG_FWD;
     extern __shared__ __align__(128) uint8_t smem[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int g = lane >> 2, t4 = lane & 3;
@@ -126,15 +120,7 @@ __global__ void __launch_bounds__(kNT, 2) k_dagg_tc(const AggArgs a, int bands_p
     const int nchunks = (D + N - 1) / N;
     float *sI = reinterpret_cast<float *>(smem + S::sI);
     float *sB = reinterpret_cast<float *>(smem + S::sB);
-    // the exponent of h's scale: |h| <= max|dS/dl| D / T, brought below 2^15
-    int hs = 0;
-    if constexpr (TWO) {
-        static_assert(kAggRange == 64, "two per lane");
-        const unsigned m = __reduce_max_sync(0xffffffffu, max(a.range[b * 64 + lane], a.range[b * 64 + 32 + lane]));
-        const int e = max((int)(m >> 23) - 127, -126) + 1 + min(ilogbf(a.invT * (float)D), 200) + 1;
-        hs = max(-126, min(126, 15 - e));
-    }
-    constexpr int vs = kAggCostShift;
+    const int hs = h_shift(a, b, lane);
     const float *img = a.img + b * HW;
     int *bad = reinterpret_cast<int *>(smem + S::bad);
     for (int i = tid; i < RR; i += kNT) bad[i] = 0;
@@ -151,7 +137,7 @@ __global__ void __launch_bounds__(kNT, 2) k_dagg_tc(const AggArgs a, int bands_p
         const int d0 = ch * N, dn = min(N, D - d0);
         const int tag0 = 1 + ch * 4 * (nsteps + 1);      // ring row cr of this chunk has the tag tag0 + cr
         const int ng = (dn + 3) / 4;
-        const __half *vol = a.vol + ((size_t)b * ((D + 3) / 4) + d0 / 4) * HW * 8;
+        const __half *vol = reinterpret_cast<const __half *>(a.vol) + ((size_t)b * ((D + 3) / 4) + d0 / 4) * HW * 8;
         {
             const int px0 = 4 * warp, mx = g & 3, my0 = g >> 2;
             // spatial exponents -(kx + 14) of this lane's columns 2 t4 + {0, 1} and + {8, 9} of a window
@@ -167,7 +153,6 @@ __global__ void __launch_bounds__(kNT, 2) k_dagg_tc(const AggArgs a, int bands_p
 #pragma unroll
             for (int j = 0; j < N / 16; ++j)
                 bo[j] = smem_addr(smem) + (uint32_t)(xq * N * 2 + (((2 * j + (lane >> 4)) ^ swz(xq)) << 4));
-            const uint32_t one = g == 0 ? 0x3c003c00u : 0u;   // the column of ones (column 0 of its tile)
             const float2 *kyl = kyt + 3 - my0;
             int slot0 = 0, slot = 0;               // ring slots of the step's first row, of the band's
             for (int p = 0; p <= nsteps; ++p) {
@@ -181,8 +166,8 @@ __global__ void __launch_bounds__(kNT, 2) k_dagg_tc(const AggArgs a, int bands_p
                         const int y = Y0 - RB + scr, u = x0 - RB + sx;
                         if (sx < QW && y >= 0 && y < H && u >= 0 && u < W) {
                             si = img[(size_t)y * W + u];
-                            if constexpr (MODE == AGG_GC) sbv = a.beta[b * HW + (size_t)y * W + u];
-                            rowbad = a.bad[b * H + y];
+                            sbv = a.beta[b * HW + (size_t)y * W + u];
+                            rowbad = a.hbad[b * H + y];
                         }
                     }
                     // warp: row r, groups wq + 2 i; lane: 8 bytes (hi or lo) of positions (lane >> 1) + 16 k
@@ -211,34 +196,21 @@ __global__ void __launch_bounds__(kNT, 2) k_dagg_tc(const AggArgs a, int bands_p
                     const int s0 = (slot + RB + my0) % RR, s2 = (slot + RB + my0 + 2) % RR;
                     const float ip0 = sI[s0 * kSIP + px0 + RB + mx], ip1 = sI[s2 * kSIP + px0 + RB + mx];
                     const float2 np0 = make_float2(-ip0, -ip0), np1 = make_float2(-ip1, -ip1);
-                    float acc[N / 8][4], ac1[TWO ? N / 8 : 1][4], zc[4], sc[4];
+                    float acc[N / 8][4], ac1[N / 8][4];
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
-                        zc[k] = sc[k] = 0.f;
 #pragma unroll
                         for (int n = 0; n < N / 8; ++n) {
-                            acc[n][k] = 0.f;
-                            if constexpr (TWO) ac1[n][k] = 0.f;
+                            acc[n][k] = ac1[n][k] = 0.f;
                         }
                     }
-                    // what the epilogue reads, asked for ahead of the products: H's three values of the two pixels;
-                    // GC's costs (lane: a group and a row of the patch) into the caches
-                    float pgl[2], plse[2], plbar[2];
-                    if constexpr (MODE == AGG_H) {
+                    // the costs that the epilogue reads, into the caches ahead of the products (lane: a disparity)
+                    if (lane < dn && x0 + px0 < W) {
+                        const float *c = a.cost + ((size_t)b * D + d0 + lane) * HW + x0 + px0;
 #pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            const int u = x0 + px0 + mx, y = Y0 + 4 * band + my0 + 2 * h;
-                            const bool in = u < W && y < H;
-                            const size_t o = b * HW + (in ? (size_t)y * W + u : 0);
-                            pgl[h] = in ? a.gdisp[o] : 0.f;
-                            plse[h] = in ? a.lse[o] : 0.f;
-                            plbar[h] = in ? a.lbar[o] : 0.f;
-                        }
-                    } else if constexpr (MODE == AGG_GC) {
-                        const int u = x0 + px0, y = Y0 + 4 * band + (lane & 3), gr = lane >> 2;
-                        if (u < W && y < H && gr < ng)
-                            asm volatile("prefetch.global.L1 [%0];" ::"l"(
-                                a.cost + (((size_t)b * ((D + 3) / 4) + d0 / 4 + gr) * HW + (size_t)y * W + u) * 8));
+                        for (int k = 0; k < 4; ++k)
+                            if (Y0 + 4 * band + k < H)
+                                asm volatile("prefetch.global.L1 [%0];" ::"l"(c + (size_t)(Y0 + 4 * band + k) * W));
                     }
                     int rs = slot + lane;
                     if (rs >= RR) rs -= RR;
@@ -251,7 +223,7 @@ __global__ void __launch_bounds__(kNT, 2) k_dagg_tc(const AggArgs a, int bands_p
                         // the weights of window row r as A fragments (hi, lo; of w, and of w t with t = sI_q - sI_p):
                         // w 2^14 = 2^-(t^2 - (kx + ky) - 14)
                         struct Frag {
-                            uint32_t ah[4], al[4], dh[TWO ? 4 : 1], dl[TWO ? 4 : 1];
+                            uint32_t ah[4], al[4], dh[4], dl[4];
                             uint32_t ro;          // the row's offset in the ring
                         };
                         auto weights = [&](Frag &f) {
@@ -266,13 +238,10 @@ __global__ void __launch_bounds__(kNT, 2) k_dagg_tc(const AggArgs a, int bands_p
                                 const float2 e = __ffma2_rn(t, t, __fadd2_rn(nk, ky));
                                 const float2 w = make_float2(ex2_approx(-e.x), ex2_approx(-e.y));
                                 split2(w.x, w.y, f.ah[i], f.al[i]);
-                                if constexpr (TWO) {
-                                    const float2 d = __fmul2_rn(w, t);                 // w (sI_q - sI_p)
-                                    split2(d.x, d.y, f.dh[i], f.dl[i]);
-                                    if constexpr (MODE == AGG_GC)
-                                        sb[i & 1] = __ffma2_rn(d, *reinterpret_cast<const float2 *>(irow + (S::sB - S::sI) / 4 + (i & 2) * 4),
-                                                               sb[i & 1]);
-                                }
+                                const float2 d = __fmul2_rn(w, t);                 // w (sI_q - sI_p)
+                                split2(d.x, d.y, f.dh[i], f.dl[i]);
+                                sb[i & 1] = __ffma2_rn(d, *reinterpret_cast<const float2 *>(irow + (S::sB - S::sI) / 4 + (i & 2) * 4),
+                                                       sb[i & 1]);
                             };
                             pairw(qlo, np0, nkx_lo, ky0, 0);
                             pairw(qlo, np1, nkx_lo, ky1, 1);
@@ -295,17 +264,11 @@ __global__ void __launch_bounds__(kNT, 2) k_dagg_tc(const AggArgs a, int bands_p
                             };
                             next();
                             pass(f.ah, vh, acc);
-                            if constexpr (TWO) pass(f.dh, vh, ac1);
+                            pass(f.dh, vh, ac1);
                             pass(f.al, vh, acc);
-                            if constexpr (TWO) pass(f.dl, vh, ac1);
+                            pass(f.dl, vh, ac1);
                             pass(f.ah, vl, acc);
-                            if constexpr (TWO) pass(f.dh, vl, ac1);
-                            if constexpr (MODE != AGG_GC) {
-                                mma(zc, f.ah, one, one);
-                                if constexpr (TWO) mma(sc, f.dh, one, one);
-                                mma(zc, f.al, one, one);
-                                if constexpr (TWO) mma(sc, f.dl, one, one);
-                            }
+                            pass(f.dh, vl, ac1);
                         };
                         Frag f0, f1;
                         weights(f0);
@@ -331,10 +294,7 @@ __global__ void __launch_bounds__(kNT, 2) k_dagg_tc(const AggArgs a, int bands_p
 #pragma unroll
                             for (int hh = 0; hh < 2; ++hh) {
                                 if (h != hh) continue;
-                                zc[2 * hh] += w;
-                                if constexpr (MODE == AGG_H) sc[2 * hh] = fmaf(w, t, sc[2 * hh]);
-                                if constexpr (MODE == AGG_GC)
-                                    if (t4 == 0) sb[hh].x = fmaf(w * t, a.beta[b * HW + (size_t)y * W + u], sb[hh].x);
+                                if (t4 == 0) sb[hh].x = fmaf(w * t, a.beta[b * HW + (size_t)y * W + u], sb[hh].x);
 #pragma unroll
                                 for (int n = 0; n < N / 8; ++n) {
                                     if (2 * n + (t4 >> 1) >= ng) continue;
@@ -342,10 +302,8 @@ __global__ void __launch_bounds__(kNT, 2) k_dagg_tc(const AggArgs a, int bands_p
                                     const float2 v = unsplit2(z[0], z[2]);
                                     acc[n][2 * hh] = fmaf(w, v.x, acc[n][2 * hh]);
                                     acc[n][2 * hh + 1] = fmaf(w, v.y, acc[n][2 * hh + 1]);
-                                    if constexpr (TWO) {
-                                        ac1[n][2 * hh] = fmaf(w * t, v.x, ac1[n][2 * hh]);
-                                        ac1[n][2 * hh + 1] = fmaf(w * t, v.y, ac1[n][2 * hh + 1]);
-                                    }
+                                    ac1[n][2 * hh] = fmaf(w * t, v.x, ac1[n][2 * hh]);
+                                    ac1[n][2 * hh + 1] = fmaf(w * t, v.y, ac1[n][2 * hh + 1]);
                                 }
                             }
                         }
@@ -358,123 +316,30 @@ __global__ void __launch_bounds__(kNT, 2) k_dagg_tc(const AggArgs a, int bands_p
                         const bool in = u < W && y < H;
                         const size_t pix = in ? (size_t)y * W + u : 0, o = b * HW + pix;
                         const bool last = ch + 1 == nchunks;
-                        if constexpr (MODE == AGG_FWD) {
-                            const float Z = __shfl_sync(0xffffffffu, zc[2 * h], lane & ~3);
-                            const float kz = -a.kT * pow2i(-vs) / Z;
-                            float m = -INFINITY, s0 = 0.f, s1 = 0.f;
+                        const float us = pow2i(-hs) * pow2i(-kWSh);
+                        float tacc = 0.f;
+                        const size_t vo = ((size_t)b * D + d0 + 2 * t4) * HW + pix;
+                        const float *cp = a.cost + vo;
+                        float cx[N / 8][2];
 #pragma unroll
-                            for (int n = 0; n < N / 8; ++n)
+                        for (int n = 0; n < N / 8; ++n)
 #pragma unroll
-                                for (int e = 0; e < 2; ++e)
-                                    if (8 * n + 2 * t4 + e < dn) m = fmaxf(m, acc[n][2 * h + e] * kz);
-                            m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));
-                            m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 2));
-                            float m0 = -INFINITY, a0 = 0.f, a1 = 0.f;      // the earlier chunks' state
-                            if (ch > 0 && in) {
-                                m0 = a.lse[o];
-                                a0 = a.lbar[o];
-                                a1 = a.disp[o];
-                            }
-                            m = fmaxf(m, m0);
+                            for (int e = 0; e < 2; ++e)
+                                cx[n][e] = in && 8 * n + 2 * t4 + e < dn ? cp[(size_t)(8 * n + e) * HW] : 0.f;
 #pragma unroll
-                            for (int n = 0; n < N / 8; ++n)
+                        for (int n = 0; n < N / 8; ++n)
 #pragma unroll
-                                for (int e = 0; e < 2; ++e)
-                                    if (8 * n + 2 * t4 + e < dn) {
-                                        const float x = ex2_approx(fmaf(acc[n][2 * h + e], kz, -m));
-                                        s0 += x;
-                                        s1 = fmaf((float)(d0 + 8 * n + 2 * t4 + e), x, s1);
-                                    }
-                            s0 = quad_sum(s0);
-                            s1 = quad_sum(s1);
-                            if (ch > 0) {
-                                const float f = exp2f(m0 - m);
-                                s0 = fmaf(a0, f, s0);
-                                s1 = fmaf(a1, f, s1);
-                            }
-                            __syncwarp();                                  // the quad has read the state
-                            if (t4 == 0 && in) {
-                                if (last) {
-                                    const float lbar = s1 / s0, sv = a.shift[(size_t)b * H + y];
-                                    a.lbar[o] = lbar;
-                                    a.lse[o] = m + log2f(s0);
-                                    a.disp[o] = lbar + (a.warp_mode == STEREO_WARP_LINEAR ? sv : round_half_up(sv));
-                                } else {
-                                    a.lse[o] = m;
-                                    a.lbar[o] = s0;
-                                    a.disp[o] = s1;
+                            for (int e = 0; e < 2; ++e)
+                                if (in && 8 * n + 2 * t4 + e < dn) {
+                                    a.gc[vo + (size_t)(8 * n + e) * HW] = acc[n][2 * h + e] * us;
+                                    tacc = fmaf(cx[n][e], ac1[n][2 * h + e], tacc);
                                 }
-                            }
-                        } else if constexpr (MODE == AGG_H) {
-                            const float Z = __shfl_sync(0xffffffffu, zc[2 * h], lane & ~3);
-                            const float S1 = __shfl_sync(0xffffffffu, sc[2 * h], lane & ~3) * pow2i(-kWSh);
-                            const float ez = pow2i(-vs) / Z, iz = pow2i(kWSh) / Z;
-                            const float gl = pgl[h], lse = plse[h], lbar = plbar[h];
-                            const float gz = -gl * a.invT * pow2i(hs);
-                            float beta = 0.f, tacc = 0.f;
-                            bool off = false;
-                            __half *hp = a.h + (((size_t)b * ((D + 3) / 4) + d0 / 4 + (t4 >> 1)) * HW + pix) * 8 + 2 * (t4 & 1);
-#pragma unroll
-                            for (int n = 0; n < N / 8; ++n) {
-                                if (!in || 2 * n + (t4 >> 1) >= ng) continue;
-                                float hv[2];
-#pragma unroll
-                                for (int e = 0; e < 2; ++e) {
-                                    const float E = acc[n][2 * h + e] * ez;
-                                    const float P = ex2_approx(-E * a.kT - lse);
-                                    const float z = gz * P * ((float)(d0 + 8 * n + 2 * t4 + e) - lbar) * iz;
-                                    hv[e] = 8 * n + 2 * t4 + e < dn ? z : 0.f;
-                                    beta = fmaf(hv[e], E, beta);
-                                    tacc = fmaf(hv[e], ac1[n][2 * h + e], tacc);
-                                    off |= off_range(hv[e]);
-                                }
-                                uint32_t hi, lo;
-                                split2(hv[0], hv[1], hi, lo);
-                                uint32_t *z = reinterpret_cast<uint32_t *>(hp + (size_t)n * HW * 16);
-                                z[0] = hi;
-                                z[2] = lo;
-                            }
-                            if (off) a.hbad[b * H + y] = 1;
-                            beta = quad_sum(beta) * pow2i(-hs);
-                            tacc = quad_sum(tacc) * pow2i(-vs - kWSh) * pow2i(-hs);
-                            if (ch > 0 && in) {
-                                beta += a.beta[o];
-                                tacc += a.t1[o];
-                            }
-                            __syncwarp();
-                            if (t4 == 0 && in) {
-                                a.beta[o] = beta;
-                                a.t1[o] = last ? fmaf(-beta, S1, tacc) : tacc;
-                            }
-                        } else {
-                            const float us = pow2i(-hs) * pow2i(-kWSh);
-                            float tacc = 0.f;
-                            const size_t vo = ((size_t)b * D + d0 + 2 * t4) * HW + pix;
-                            const uint32_t *cp = reinterpret_cast<const uint32_t *>(
-                                a.cost + (((size_t)b * ((D + 3) / 4) + d0 / 4 + (t4 >> 1)) * HW + pix) * 8 + 2 * (t4 & 1));
-                            uint32_t ch_[N / 8], cl_[N / 8];
-#pragma unroll
-                            for (int n = 0; n < N / 8; ++n) {
-                                ch_[n] = in && 2 * n + (t4 >> 1) < ng ? cp[(size_t)n * HW * 8] : 0u;
-                                cl_[n] = in && 2 * n + (t4 >> 1) < ng ? cp[(size_t)n * HW * 8 + 2] : 0u;
-                            }
-#pragma unroll
-                            for (int n = 0; n < N / 8; ++n) {
-                                const float2 c = unsplit2(ch_[n], cl_[n]);
-#pragma unroll
-                                for (int e = 0; e < 2; ++e)
-                                    if (in && 8 * n + 2 * t4 + e < dn) {
-                                        a.gc[vo + (size_t)(8 * n + e) * HW] = acc[n][2 * h + e] * us;
-                                        tacc = fmaf(e ? c.y : c.x, ac1[n][2 * h + e], tacc);
-                                    }
-                            }
-                            tacc = quad_sum(tacc) * us * pow2i(-vs);
-                            const float sbh = quad_sum(sb[h].x + sb[h].y) * pow2i(-kWSh);
-                            if (ch == 0) tacc -= sbh;
-                            else if (in) tacc += a.gw[o];
-                            __syncwarp();
-                            if (t4 == 0 && in) a.gw[o] = last ? a.gw_scale * (a.t1[o] + tacc) : tacc;
-                        }
+                        tacc = quad_sum(tacc) * us;
+                        const float sbh = quad_sum(sb[h].x + sb[h].y) * pow2i(-kWSh);
+                        if (ch == 0) tacc -= sbh;
+                        else if (in) tacc += a.gw[o];
+                        __syncwarp();
+                        if (t4 == 0 && in) a.gw[o] = last ? a.gw_scale * (a.t1[o] + tacc) : tacc;
                     }
                 }
                 if (p < nsteps && sr < 4 && scr >= 0) {
@@ -482,7 +347,7 @@ __global__ void __launch_bounds__(kNT, 2) k_dagg_tc(const AggArgs a, int bands_p
                     if (sl >= RR) sl -= RR;
                     if (si != kFar) si *= a.kappa;
                     sI[sl * kSIP + sx] = si;
-                    if constexpr (MODE == AGG_GC) sB[sl * kSIP + sx] = sbv;
+                    sB[sl * kSIP + sx] = sbv;
                     if (rowbad || !(fabsf(si) <= kFar && fabsf(sbv) < INFINITY)) bad[sl] = tag0 + scr;
                 }
                 slot0 += 4 * p - S::PHI + 4 - first;
@@ -498,7 +363,7 @@ __global__ void __launch_bounds__(kNT, 2) k_dagg_tc(const AggArgs a, int bands_p
     }
 }
 
-template <int MODE, int RB>
+template <int RB>
 cudaError_t launch_rb(const AggArgs &a, int B, cudaStream_t st)
 {
     using S = Shape<RB>;
@@ -506,7 +371,7 @@ cudaError_t launch_rb(const AggArgs &a, int B, cudaStream_t st)
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_dagg_tc<MODE, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::total);
+        e = cudaFuncSetAttribute(k_dagg_tc<RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::total);
     if (e != cudaSuccess) return e;
     // bands per segment: of all equal splits, the one whose waves (one CTA per SM) take the fewest
     // iterations
@@ -521,32 +386,29 @@ cudaError_t launch_rb(const AggArgs &a, int B, cudaStream_t st)
             best = nb;
         }
     }
-    k_dagg_tc<MODE, RB><<<dim3(strips * ((bands + best - 1) / best), B), kNT, S::total, st>>>(a, best);
+    k_dagg_tc<RB><<<dim3(strips * ((bands + best - 1) / best), B), kNT, S::total, st>>>(a, best);
     return cudaGetLastError();
-}
-
-template <int MODE>
-cudaError_t launch_mode(const AggArgs &a, int rb, int B, cudaStream_t st)
-{
-    switch (rb) {
-#define SGB_AGG(R) case R: return launch_rb<MODE, R>(a, B, st);
-    SGB_AGG(0) SGB_AGG(1) SGB_AGG(2) SGB_AGG(3) SGB_AGG(4) SGB_AGG(5)
-#undef SGB_AGG
-    default: return launch_rb<MODE, 6>(a, B, st);
-    }
 }
 
 }  // namespace
 
-cudaError_t launch_agg_tc(int mode, const AggArgsT<__half> &a, int rb, int B, cudaStream_t st)
+cudaError_t launch_dabsmax(const AggArgs &a, int B, cudaStream_t st)
 {
-    if (mode == AGG_FWD) return launch_mode<AGG_FWD>(a, rb, B, st);
-    if (mode == AGG_H) {
-        k_dabsmax<<<dim3(kAggRange, B), 256, 0, st>>>(a.gdisp, a.H, a.W, a.range, a.hbad);
-        const cudaError_t e = cudaGetLastError();
-        return e != cudaSuccess ? e : launch_mode<AGG_H>(a, rb, B, st);
+    k_dabsmax<<<dim3(kAggRange, B), 256, 0, st>>>(a.gdisp, a.H, a.W, a.range, a.hbad);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_gc_tc(const AggArgs &a, int rb, int B, cudaStream_t st)
+{
+    switch (rb) {
+    case 0: return launch_rb<0>(a, B, st);
+    case 1: return launch_rb<1>(a, B, st);
+    case 2: return launch_rb<2>(a, B, st);
+    case 3: return launch_rb<3>(a, B, st);
+    case 4: return launch_rb<4>(a, B, st);
+    case 5: return launch_rb<5>(a, B, st);
+    default: return launch_rb<6>(a, B, st);
     }
-    return launch_mode<AGG_GC>(a, rb, B, st);
 }
 
 }  // namespace sgb

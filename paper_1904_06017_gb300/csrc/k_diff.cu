@@ -1,24 +1,23 @@
 // k_diff.cu -- soft-argmin disparity over the bilateral-aggregated cost and its adjoint
-// (include/stereo_diff.h).  FP32 throughout, but that the cost volume and h are held, up to bil = 13,
-// as pairs of FP16 halves (22 bits, k_diff.cuh) for the tensor-core form of the aggregation.  The
-// aggregated volume E(p,d) of eq. (fbs) is never stored: the backward pass recomputes it from the stored
-// cost volume.
+// (include/stereo_diff.h).  FP32 throughout (but that h goes from H to GC, up to bil = 13, as pairs of FP16
+// halves, 22 bits: k_diff.cuh); the aggregated volume E(p,d) of eq. (fbs) is
+// never stored: the backward pass recomputes it tile by tile from the stored cost volume.
 //
 // Forward (per pair of a batch, float images):
 //   k_dwarp     tw(u,v) = tgt(clamp(u - s_i(v)), v)                                   §3.1
 //   k_dstats    window mean / population std of ref (image grid) and of tw (columns
 //               shifted by -(D-1), so that the target window of (p, d) is the entry at u-d)
 //   k_dcost     c(p,d) = 1 - sum_i (a_i - mu_a)(b_i - mu_b) / (n s_a s_b)           eq. (c)
-//   agg FWD     E(p,d) = sum_q w c / sum_q w (eq. omega_s, eq. fbs), online soft-max over d:
+//   k_dagg<FWD> E(p,d) = sum_q w c / sum_q w (eq. omega_s, eq. fbs), online soft-max over d:
 //               l = sum_d d P(p,d) + s_i(v), P = softmax_d(-E/T); keeps log2-sum-exp, lbar
-//               (k_dagg_tc.cu up to bil = 13, k_dagg here at 15)
 // Backward, given gl = dS/dl:
 //   k_dabsmax   the scale of h, from max |gl| of each image
-//   agg H       recompute E; gE = -gl P (d - lbar) / T; h = gE / Z(p);  beta(p) = sum_d h E;
+//   k_dagg<H>   recompute E; gE = -gl P (d - lbar) / T; h = gE / Z(p);  beta(p) = sum_d h E;
 //               t1(p) = sum_d h(p,d) sum_q w (I_q - I_p) c(q,d) - beta(p) sum_q w (I_q - I_p)
 //   agg GC      gc(q,d) = sum_p w(p,q) h(p,d)                  (adjoint of eq. fbs in c)
 //               gw(x) = 2/sigma1^2 (t1(x) + sum_d c(x,d) sum_q w (I_q - I_x) h(q,d)
 //                                        - sum_q w (I_q - I_x) beta(q))  (through the weights)
+//               (k_dagg_tc.cu up to bil = 13, k_dagg<GC> here at 15)
 //   k_dcost_bwd adjoint of eq. (c).  Per window pair (q, d), with g = gc(q,d) / n and the target
 //               block qt = q - d:  A = -g / (s_a s_b),  B = g ncc / s_a^2,  C = g ncc / s_b^2;
 //               an extended reference position X collects
@@ -47,6 +46,7 @@
 
 namespace sgb {
 namespace {
+
 
 // pixels per thread in k_dagg (a column segment): the forward pass, with one accumulator set,
 // takes 8, so that each staged neighbour row serves twice the weights
@@ -107,8 +107,8 @@ struct Dims {
 struct Ws {
     float *tw, *mur, *sdr, *mut, *isdt, *cost, *lse, *lbar;      // forward (isdt: 1 / s_b, 0 where flat)
     float *h, *gc, *beta, *t1, *gw, *gpart, *gqpart, *samb, *sb, *grefx, *gtwx;      // backward
-    unsigned *range;               // split volumes: scale of h, rows that the split cannot carry
-    int *cbad, *hbad;
+    unsigned *range;               // split h: its scale, and the rows that the split cannot carry
+    int *hbad;
 };
 
 size_t layout(const Dims &d, char *base, Ws *w)
@@ -118,7 +118,8 @@ size_t layout(const Dims &d, char *base, Ws *w)
         if (p) *p = base ? (float *)(base + off) : nullptr;
         off += (elems * sizeof(float) + 255) / 256 * 256;
     };
-    const size_t B = d.B, img = (size_t)d.H * d.W, vol = (size_t)((d.D + 3) / 4 * 4) * img;   // (groups of 4: split layout)
+    const size_t B = d.B, img = (size_t)d.H * d.W, vol = (size_t)d.D * img,
+                 volh = (size_t)((d.D + 3) / 4 * 4) * img;   // (h: groups of 4 in the split layout)
     Ws tmp;
     Ws *o = w ? w : &tmp;
     take(&o->tw, B * img);
@@ -129,18 +130,20 @@ size_t layout(const Dims &d, char *base, Ws *w)
     take(&o->cost, B * vol);
     take(&o->lse, B * img);
     take(&o->lbar, B * img);
-    take(&o->h, B * vol);
+    // h, and in its place once it has been read the cost adjoint's sums along q - d
+    const size_t gq = (2 * B * (size_t)d.H * cb_tiles_x(d.Wr) * cb_diag_w(d.D) + 63) / 64 * 64, im = (B * img + 63) / 64 * 64;
+    const size_t share = gq + 2 * im;
+    take(&o->h, B * volh > share ? B * volh : share);
+    o->gqpart = o->h;
+    o->samb = o->h ? o->h + gq : nullptr;
+    o->sb = o->h ? o->h + gq + im : nullptr;
     take(&o->gc, B * vol);
     take(&o->beta, B * img);
     take(&o->t1, B * img);
     take(&o->gw, B * img);
     take(&o->gpart, B * (size_t)d.Hr * cb_tiles_x(d.Wr) * cb_diag_w(d.D));
-    take(&o->gqpart, 2 * B * (size_t)d.H * cb_tiles_x(d.Wr) * cb_diag_w(d.D));
     take((float **)&o->range, B * kAggRange);
-    take((float **)&o->cbad, B * (size_t)d.H);
     take((float **)&o->hbad, B * (size_t)d.H);
-    take(&o->samb, B * img);
-    take(&o->sb, B * img);
     take(&o->grefx, B * (size_t)d.Hr * d.Wr);
     take(&o->gtwx, B * (size_t)d.Hr * d.Wt);
     return off;
@@ -211,11 +214,10 @@ __device__ __forceinline__ LinShift lin_shift(float s, int W)
 }
 
 __global__ void __launch_bounds__(256) k_dwarp(const float *__restrict__ tgt, const float *__restrict__ shift,
-                                               float *__restrict__ tw, int *__restrict__ cbad, int W, int H, int mode)
+                                               float *__restrict__ tw, int W, int H, int mode)
 {
     const int u = blockIdx.x * blockDim.x + threadIdx.x, v = blockIdx.y, b = blockIdx.z;
     if (u >= W) return;
-    if (u == 0) cbad[b * H + v] = 0;   // set by k_dcost
     const size_t row = ((size_t)b * H + v) * W;
     const float s = shift[(size_t)b * H + v];
     if (mode == STEREO_WARP_LINEAR) {
@@ -320,8 +322,7 @@ template <int RW>
 __global__ void __launch_bounds__(kCostThreads, 3) k_dcost(const float *__restrict__ ref, const float *__restrict__ tw,
                                                   const float *__restrict__ mur, const float *__restrict__ sdr,
                                                   const float *__restrict__ mut, const float *__restrict__ isdt,
-                                                  float *__restrict__ cost, int *__restrict__ cbad, int split, int W, int H,
-                                                  int D, int nchunk)
+                                                  float *__restrict__ cost, int W, int H, int D, int nchunk)
 {
     constexpr int DC = kCostDC, rw = RW, w = 2 * RW + 1;
     constexpr int PRW = dcost_rw_pairs(RW), PTW = dcost_tw_pairs(RW), SH = dcost_rows(RW);
@@ -448,37 +449,16 @@ __global__ void __launch_bounds__(kCostThreads, 3) k_dcost(const float *__restri
             const int u = u0 + 32 * j, v = v0 + h;
             const float sav = sdr[b * HW + (size_t)v * W + u], as = j ? asum[h].y : asum[h].x;
             const float ia = sav > 0.f ? 1.f / (n * sav) : 0.f;   // 1 / (n s_a), once per pixel
-            auto value = [&](int k) {
+#pragma unroll
+            for (int k = 0; k < DC; ++k) {
+                const int d = d0 + k;
+                if (d >= D) break;
                 const int e = (2 * ty + h) * kCostSW + tx + 32 * j - k + DC - 1;
                 const float mb = smb[e], isb = ssb[e];
                 const float ak = j ? acc[h][k].y : acc[h][k].x;
-                return ia > 0.f && isb > 0.f ? 1.f - fmaf(-mb, as, ak) * ia * isb : 1.f;
-            };
-            const size_t pix = (size_t)v * W + u;
-            if (split) {
-                bool off = false;
-#pragma unroll
-                for (int gr = 0; gr < DC / 4; ++gr) {
-                    if (d0 + 4 * gr >= D) break;
-                    uint32_t hi[2], lo[2];
-#pragma unroll
-                    for (int k = 0; k < 2; ++k) {
-                        const int d = d0 + 4 * gr + 2 * k;
-                        const float c0 = d < D ? value(4 * gr + 2 * k) * (float)(1 << kAggCostShift) : 0.f;
-                        const float c1 = d + 1 < D ? value(4 * gr + 2 * k + 1) * (float)(1 << kAggCostShift) : 0.f;
-                        off |= off_range(c0) | off_range(c1);
-                        split2(c0, c1, hi[k], lo[k]);
-                    }
-                    reinterpret_cast<uint4 *>(cost)[((size_t)b * ((D + 3) / 4) + d0 / 4 + gr) * HW + pix] =
-                        make_uint4(hi[0], hi[1], lo[0], lo[1]);
-                }
-                if (off) cbad[b * H + v] = 1;
-            } else {
-#pragma unroll
-                for (int k = 0; k < DC; ++k) {
-                    if (d0 + k >= D) break;
-                    cost[((size_t)b * D + d0 + k) * HW + pix] = value(k);
-                }
+                float c = 1.f;
+                if (ia > 0.f && isb > 0.f) c = 1.f - fmaf(-mb, as, ak) * ia * isb;
+                cost[((size_t)b * D + d) * HW + (size_t)v * W + u] = c;
             }
         }
 }
@@ -503,8 +483,6 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 // i < R = agg_rows(MODE), and kAggDC disparities at a time.  The weights of eq. (omega_s) are formed as
 // exp2(kx + ky - (sI_p - sI_q)^2) with sI = kappa I; an out-of-image neighbour has
 // sI = kFar and a zero value, so its weight and every product with it are exactly 0.
-using AggArgs = AggArgsT<float>;
-
 template <int MODE, int RB>
 __global__ void __launch_bounds__(agg_threads(MODE), MODE == AGG_FWD ? 3 : MODE == AGG_GC ? 2 : 1) k_dagg(const AggArgs a)
 {
@@ -514,6 +492,7 @@ __global__ void __launch_bounds__(agg_threads(MODE), MODE == AGG_FWD ? 3 : MODE 
     constexpr int kAggTX = agg_tx(MODE), kAggTY = agg_ty(MODE), kAggThreads = agg_threads(MODE);
     constexpr int TW = kAggTX + 2 * RB, TH = kAggTY + 2 * RB;
     constexpr bool TWO = MODE != AGG_FWD;
+    constexpr bool SPLIT = MODE == AGG_H && RB <= kAggTcMaxRB;     // h goes to k_dagg_tc
     extern __shared__ float4 smem4[];
     float4 *Vbuf = smem4;                                     // [1 or 2][NQ][TH][TW]
     float *sI = (float *)(Vbuf + (DB ? 2 : 1) * NQ * TH * TW); // [TH][TW]
@@ -569,6 +548,8 @@ __global__ void __launch_bounds__(agg_threads(MODE), MODE == AGG_FWD ? 3 : MODE 
             if (i < TH * TW) sI[i] = vi[it];
         }
     }
+    float hscale = 1.f;
+    if constexpr (SPLIT) hscale = pow2i(h_shift(a, b, threadIdx.x & 31));
     float ky[2 * RB + 1];
 #pragma unroll
     for (int j = 0; j <= 2 * RB; ++j) ky[j] = a.k0 * (float)((j - RB) * (j - RB));
@@ -710,16 +691,36 @@ __global__ void __launch_bounds__(agg_threads(MODE), MODE == AGG_FWD ? 3 : MODE 
                 st1[i] = s0;
                 st2[i] = s1;
             } else if constexpr (MODE == AGG_H) {
+                float hk[DC];
 #pragma unroll
                 for (int k = 0; k < DC; ++k) {
                     const int d = d0 + k;
-                    if (d >= D) break;
+                    hk[k] = 0.f;
+                    if (d >= D) continue;
                     const float E = lane(acc0[i][k >> 1], k) * invZ[i];
                     const float P = exp2f(-E * a.kT - st1[i]);
                     const float hv = -st0[i] * a.invT * P * ((float)d - st2[i]) * invZ[i];
-                    a.h[((size_t)b * D + d) * HW + pix] = hv;
+                    if constexpr (!SPLIT) a.h[((size_t)b * D + d) * HW + pix] = hv;
+                    hk[k] = hv;
                     beta[i] = fmaf(hv, E, beta[i]);
                     tacc[i] = fmaf(hv, lane(acc1[i][k >> 1], k), tacc[i]);
+                }
+                if constexpr (SPLIT) {
+                    bool off = false;
+#pragma unroll
+                    for (int q = 0; q < DC / 4; ++q) {
+                        if (d0 + 4 * q >= D) break;
+                        uint4 v;
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            hk[4 * q + k] *= hscale;
+                            off |= off_range(hk[4 * q + k]);
+                        }
+                        split2(hk[4 * q], hk[4 * q + 1], v.x, v.z);
+                        split2(hk[4 * q + 2], hk[4 * q + 3], v.y, v.w);
+                        reinterpret_cast<uint4 *>(a.h)[((size_t)b * ((D + 3) / 4) + d0 / 4 + q) * HW + pix] = v;
+                    }
+                    if (off) a.hbad[b * H + py[i]] = 1;
                 }
             } else {
 #pragma unroll
@@ -805,7 +806,6 @@ __global__ void __launch_bounds__(agg_threads(MODE), MODE == AGG_FWD ? 3 : MODE 
 // ------------------------------------------------------------------ cost adjoint
 struct CbArgs {
     const float *ref, *tw, *mur, *sdr, *mut, *isdt, *cost, *gc;
-    int split;             // cost is a split volume
     float *gpart;          // [B][Hr][tile column][32 + D - 1] partial sums over X of r(X) bA(X, d) (or null)
     float2 *gqpart;        // [B][H][tile column][32 + D - 1] partial sums over q of (A mu_a, C) (or null)
     float *samb, *sb;      // [B][H][W] sum_d A mu_b, sum_d B
@@ -929,9 +929,7 @@ __global__ void __launch_bounds__(256, 2) k_dcost_bwd(const CbArgs a)
     // previous round's box sums run
     const float *gcb = a.gc + (size_t)b * D * HW, *cob = a.cost + (size_t)b * D * HW;
     const float *isb = a.isdt + (size_t)b * H * a.We, *mub = a.mut + (size_t)b * H * a.We;
-    float g[NS][DC], sbv[NS][DC], mb[NO][DC];
-    uint4 cc[NO];          // the costs as they are stored: four floats, or a group of the split volume
-    static_assert(DC == 4, "a group of the split cost volume");
+    float g[NS][DC], sbv[NS][DC], cc[NO][DC], mb[NO][DC];
     auto load_round = [&](int d0) {
 #pragma unroll
         for (int k = 0; k < DC; ++k) {
@@ -944,15 +942,10 @@ __global__ void __launch_bounds__(256, 2) k_dcost_bwd(const CbArgs a)
                 g[s][k] = ok ? gp[qo[s]] : 0.f;
                 sbv[s][k] = ok ? isb[sk] : 0.f;   // 1 / s_b (0: a flat target block)
                 if (s < NO) {
-                    if (!a.split) (&cc[s].x)[k] = ok ? __float_as_uint(cp[qo[s]]) : 0u;
+                    cc[s][k] = ok ? cp[qo[s]] : 1.f;
                     mb[s][k] = ok ? mub[sk] - lev.y : 0.f;
                 }
             }
-        }
-        if (a.split) {
-            const uint4 *cg = reinterpret_cast<const uint4 *>(a.cost) + ((size_t)b * ((D + 3) / 4) + d0 / 4) * HW;
-#pragma unroll
-            for (int s = 0; s < NO; ++s) cc[s] = qin[s] ? cg[qo[s]] : make_uint4(0, 0, 0, 0);
         }
     };
     load_round(0);
@@ -963,16 +956,6 @@ __global__ void __launch_bounds__(256, 2) k_dcost_bwd(const CbArgs a)
         for (int s = 0; s < NS; ++s) {
             const int j = threadIdx.x + 256 * s;
             if (j >= NQ) break;
-            float4 cf = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (s < NO) {
-                const uint4 q = cc[s < NO ? s : 0];
-                cf = make_float4(__uint_as_float(q.x), __uint_as_float(q.y), __uint_as_float(q.z), __uint_as_float(q.w));
-                if (a.split) {
-                    const float2 v0 = unsplit2(q.x, q.z), v1 = unsplit2(q.y, q.w);
-                    const float sc = 1.f / (1 << kAggCostShift);
-                    cf = make_float4(v0.x * sc, v0.y * sc, v1.x * sc, v1.y * sc);
-                }
-            }
 #pragma unroll
             for (int k = 0; k < DC; ++k) {
                 float A = 0.f, gn = 0.f;
@@ -985,7 +968,7 @@ __global__ void __launch_bounds__(256, 2) k_dcost_bwd(const CbArgs a)
                 if (s < NO) {
                     float C = 0.f;
                     if (live) {
-                        const float gnc = gn * (1.f - (&cf.x)[k]);
+                        const float gnc = gn * (1.f - cc[s][k]);
                         sB[s] = fmaf(gnc * qisa[s], qisa[s], sB[s]);
                         C = gnc * sbv[s][k] * sbv[s][k];
                     }
@@ -1330,6 +1313,25 @@ cudaError_t launch_agg_rb(const AggArgs &a, int B, cudaStream_t st)
     return cudaGetLastError();
 }
 
+template <int MODE>
+cudaError_t launch_agg(const AggArgs &a, int rb, int B, cudaStream_t st)
+{
+    if constexpr (MODE != AGG_GC) {
+        switch (rb) {
+        case 0: return launch_agg_rb<MODE, 0>(a, B, st);
+        case 1: return launch_agg_rb<MODE, 1>(a, B, st);
+        case 2: return launch_agg_rb<MODE, 2>(a, B, st);
+        case 3: return launch_agg_rb<MODE, 3>(a, B, st);
+        case 4: return launch_agg_rb<MODE, 4>(a, B, st);
+        case 5: return launch_agg_rb<MODE, 5>(a, B, st);
+        case 6: return launch_agg_rb<MODE, 6>(a, B, st);
+        }
+    } else if (rb <= kAggTcMaxRB) {       // (k_dagg_tc.cu has both sides' times)
+        return launch_gc_tc(a, rb, B, st);
+    }
+    return launch_agg_rb<MODE, kAggTcMaxRB + 1>(a, B, st);
+}
+
 template <int RW>
 cudaError_t launch_cb_rw(const CbArgs &a, int B, cudaStream_t st)
 {
@@ -1356,10 +1358,9 @@ cudaError_t launch_cb(const CbArgs &a, int rw, int B, cudaStream_t st)
     }
 }
 
-template <class VT>
-AggArgsT<VT> agg_args(const stereo_diff_params *p, const Dims &d, const Ws &w, const float *ref)
+AggArgs agg_args(const stereo_diff_params *p, const Dims &d, const Ws &w, const float *ref)
 {
-    AggArgsT<VT> a;
+    AggArgs a;
     memset(&a, 0, sizeof(a));
     a.img = ref;
     a.W = d.W;
@@ -1373,56 +1374,7 @@ AggArgsT<VT> agg_args(const stereo_diff_params *p, const Dims &d, const Ws &w, c
     a.gw_scale = 2.0f / (p->sigma1 * p->sigma1 * a.kappa);
     a.lse = w.lse;
     a.lbar = w.lbar;
-    a.beta = w.beta;
-    a.t1 = w.t1;
-    a.gc = w.gc;
-    a.gw = w.gw;
-    a.range = w.range;
-    a.hbad = w.hbad;
     return a;
-}
-
-// One mode of the aggregation: volumes split and on the tensor cores up to bil = 13 (k_dagg_tc.cu has both
-// sides' times), FP32 (k_dagg) at 15, where a patch's window rows exceed the 16 k-slots of an mma.
-template <class VT>
-cudaError_t launch_agg(int mode, const AggArgsT<VT> &a, int rb, int B, cudaStream_t st)
-{
-    if constexpr (sizeof(VT) == 2) {
-        return launch_agg_tc(mode, a, rb, B, st);
-    } else {
-        if (mode == AGG_FWD) return launch_agg_rb<AGG_FWD, kAggTcMaxRB + 1>(a, B, st);
-        if (mode == AGG_H) return launch_agg_rb<AGG_H, kAggTcMaxRB + 1>(a, B, st);
-        return launch_agg_rb<AGG_GC, kAggTcMaxRB + 1>(a, B, st);
-    }
-}
-
-template <class VT>
-cudaError_t run_agg_fwd(const stereo_diff_params *p, const Dims &d, const Ws &w, const float *ref, const float *shift,
-                        float *disp, cudaStream_t st)
-{
-    AggArgsT<VT> a = agg_args<VT>(p, d, w, ref);
-    a.vol = (const VT *)w.cost;
-    a.bad = w.cbad;
-    a.shift = shift;
-    a.disp = disp;
-    return launch_agg(AGG_FWD, a, d.rb, d.B, st);
-}
-
-template <class VT>
-cudaError_t run_agg_bwd(const stereo_diff_params *p, const Dims &d, const Ws &w, const float *ref, const float *gdisp,
-                        cudaStream_t st)
-{
-    AggArgsT<VT> a = agg_args<VT>(p, d, w, ref);
-    a.vol = (const VT *)w.cost;
-    a.bad = w.cbad;
-    a.gdisp = gdisp;
-    a.h = (VT *)w.h;
-    const cudaError_t e = launch_agg(AGG_H, a, d.rb, d.B, st);
-    if (e != cudaSuccess) return e;
-    a.vol = (const VT *)w.h;
-    a.bad = w.hbad;
-    a.cost = (const VT *)w.cost;
-    return launch_agg(AGG_GC, a, d.rb, d.B, st);
 }
 
 }  // namespace
@@ -1466,7 +1418,7 @@ extern "C" int stereo_softargmin_fwd(const stereo_diff_params *p, const float *r
     if ((rc = check_ws(d, ws, ws_bytes, &w, who))) return rc;
     cudaStream_t st = (cudaStream_t)stream;
     const int B = d.B;
-    k_dwarp<<<dim3((d.W + 255) / 256, d.H, B), 256, 0, st>>>(tgt, shift, w.tw, w.cbad, d.W, d.H, d.warp_mode);
+    k_dwarp<<<dim3((d.W + 255) / 256, d.H, B), 256, 0, st>>>(tgt, shift, w.tw, d.W, d.H, d.warp_mode);
     const size_t ssm = (size_t)(32 + 2 * d.rw) * (8 + 2 * d.rw) * sizeof(float);
     launch_dstats(d.rw, dim3((d.W + 31) / 32, (d.H + 7) / 8, B), ssm, st, ref, d.W, d.H, d.W, 0, w.mur, w.sdr,
                   nullptr);
@@ -1477,8 +1429,7 @@ extern "C" int stereo_softargmin_fwd(const stereo_diff_params *p, const float *r
     {
         const dim3 grid((d.W + kCostTX - 1) / kCostTX, (d.H + kCostTY - 1) / kCostTY, B * nchunk);
 #define SGB_DCOST(R)                                                                                  \
-    k_dcost<R><<<grid, kCostThreads, csm, st>>>(ref, w.tw, w.mur, w.sdr, w.mut, w.isdt, w.cost, w.cbad, d.rb <= kAggTcMaxRB, d.W, d.H, \
-                                                d.D, nchunk)
+    k_dcost<R><<<grid, kCostThreads, csm, st>>>(ref, w.tw, w.mur, w.sdr, w.mut, w.isdt, w.cost, d.W, d.H, d.D, nchunk)
         switch (d.rw) {
         case 0: SGB_DCOST(0); break;
         case 1: SGB_DCOST(1); break;
@@ -1493,8 +1444,11 @@ extern "C" int stereo_softargmin_fwd(const stereo_diff_params *p, const float *r
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_error(e, who);
-    e = d.rb <= kAggTcMaxRB ? run_agg_fwd<__half>(p, d, w, ref, shift, disp, st)
-                            : run_agg_fwd<float>(p, d, w, ref, shift, disp, st);
+    AggArgs a = agg_args(p, d, w, ref);
+    a.vol = w.cost;
+    a.shift = shift;
+    a.disp = disp;
+    e = launch_agg<AGG_FWD>(a, d.rb, B, st);
     return cuda_error(e, who);
 }
 
@@ -1512,8 +1466,22 @@ extern "C" int stereo_softargmin_bwd(const stereo_diff_params *p, const float *r
     if (!gref && !gtgt && !gshift) return STEREO_OK;
     cudaStream_t st = (cudaStream_t)stream;
     const int B = d.B;
-    cudaError_t e = d.rb <= kAggTcMaxRB ? run_agg_bwd<__half>(p, d, w, ref, gdisp, st)
-                                        : run_agg_bwd<float>(p, d, w, ref, gdisp, st);
+    AggArgs a = agg_args(p, d, w, ref);
+    a.vol = w.cost;
+    a.gdisp = gdisp;
+    a.h = w.h;
+    a.beta = w.beta;
+    a.t1 = w.t1;
+    a.range = w.range;
+    a.hbad = w.hbad;
+    cudaError_t e = d.rb <= kAggTcMaxRB ? launch_dabsmax(a, B, st) : cudaSuccess;
+    if (e == cudaSuccess) e = launch_agg<AGG_H>(a, d.rb, B, st);
+    if (e != cudaSuccess) return cuda_error(e, who);
+    a.vol = w.h;
+    a.gc = w.gc;
+    a.cost = w.cost;
+    a.gw = w.gw;
+    e = launch_agg<AGG_GC>(a, d.rb, B, st);
     if (e != cudaSuccess) return cuda_error(e, who);
     CbArgs c;
     c.ref = ref;
@@ -1524,7 +1492,6 @@ extern "C" int stereo_softargmin_bwd(const stereo_diff_params *p, const float *r
     c.isdt = w.isdt;
     c.cost = w.cost;
     c.gc = w.gc;
-    c.split = d.rb <= kAggTcMaxRB;
     const bool need_tw = gtgt || gshift;    // the warped-target gradient feeds both
     c.gpart = need_tw ? w.gpart : nullptr;
     c.gqpart = need_tw ? (float2 *)w.gqpart : nullptr;

@@ -8,12 +8,10 @@ namespace sgb {
 
 enum { AGG_FWD = 0, AGG_H = 1, AGG_GC = 2 };
 
-// A volume value v as FP16 halves: hi = RN16(2^k v), lo = RN16(2^k v - hi), 22 bits and 32 bits of
-// memory.  Laid out as [B][ceil(D / 4)][H][W][8]: 4 hi, then 4 lo of the group's disparities (zero
-// beyond D), so that a row of a group is one run of 16 bytes per pixel.  k is kAggCostShift for the cost
-// volume (1 - ncc, above 2 by rounding only: up to about 100 on nearly flat windows).
-constexpr int kAggCostShift = 4;
-constexpr int kAggRange = 64;
+// A value v of h as FP16 halves: hi = RN16(2^k v), lo = RN16(2^k v - hi), 22 bits and 32 bits of memory.
+// Laid out as [B][ceil(D / 4)][H][W][8]: 4 hi, then 4 lo of the group's disparities (zero beyond D), so
+// that a row of a group is one run of 16 bytes per pixel.
+constexpr int kAggRange = 64;    // partial maxima of |dS/dl| per image
 
 __device__ __forceinline__ uint32_t h2(float lo, float hi)
 {
@@ -39,23 +37,22 @@ __device__ __forceinline__ float2 unsplit2(uint32_t hi, uint32_t lo)
 // A scaled value that an FP16 pair cannot carry (infinite, NaN, or out of range).
 __device__ __forceinline__ bool off_range(float x) { return !(fabsf(x) < 65504.f); }
 
-// VT: float for the volumes of k_dagg ([B][D][H][W]), __half for split ones (k_dagg_tc).
-template <class VT>
-struct AggArgsT {
+__device__ __forceinline__ float pow2i(int k) { return __int_as_float((k + 127) << 23); }   // -126 <= k <= 127
+
+struct AggArgs {
     const float *img;      // reference image [B][H][W]
-    const VT *vol;         // neighbour values: the cost (FWD, H) or h (GC)
+    const float *vol;      // neighbour values: the cost (FWD, H) or h (GC; split up to kAggTcMaxRB) [B][D][H][W]
     const float *shift;    // FWD: row shifts
     float *disp;           // FWD: l
     float *lse, *lbar;     // FWD out, H in
     const float *gdisp;    // H: dS/dl
-    VT *h;                 // H out
+    float *h;              // H out (split up to kAggTcMaxRB)
     float *beta, *t1;      // H out, GC in
-    float *gc;             // GC out: [B][D][H][W]
-    const VT *cost;        // GC: c(x, d) of the centre pixel
+    float *gc;             // GC out
+    const float *cost;     // GC: c(x, d) of the centre pixel
     float *gw;             // GC out: image gradient through the weights
-    unsigned *range;       // split: [B][kAggRange] partial maxima of |dS/dl|, bits (H out, GC in)
-    const int *bad;        // split: [B][H] rows of vol that hold a value the split cannot carry
-    int *hbad;             // split: the same of h (H out)
+    unsigned *range;       // split h: [B][kAggRange] partial maxima of |dS/dl|, bits
+    int *hbad;             // split h: [B][H] rows of h that hold a value the split cannot carry
     int W, H, D;
     int warp_mode;         // FWD: the add-back is s_i (rounded) or s(v) (linear warp)
     float kappa;           // sqrt(log2 e) / sigma1: scaled intensities
@@ -65,9 +62,20 @@ struct AggArgsT {
     float gw_scale;        // 2 / (sigma1^2 kappa)
 };
 
+// The exponent of h's scale in image b, called by a whole warp: |h| <= max|dS/dl| D / T, brought below 2^15.
+__device__ __forceinline__ int h_shift(const AggArgs &a, int b, int lane)
+{
+    static_assert(kAggRange == 64, "two per lane");
+    const unsigned m = __reduce_max_sync(0xffffffffu, max(a.range[b * 64 + lane], a.range[b * 64 + 32 + lane]));
+    const int e = max((int)(m >> 23) - 127, -126) + 1 + min(ilogbf(a.invT * (float)a.D), 200) + 1;
+    return max(-126, min(126, 15 - e));
+}
+
 constexpr int kAggTcMaxRB = 6;   // bil <= 13: a patch's window row fits the 16 k-slots of an mma
 
-// The aggregation stencils on the tensor cores (k_dagg_tc.cu); rb <= kAggTcMaxRB.
-cudaError_t launch_agg_tc(int mode, const AggArgsT<__half> &a, int rb, int B, cudaStream_t st);
+// k_dagg_tc.cu: the partial maxima that scale h and its row flags cleared (before H); GC on the tensor
+// cores (rb <= kAggTcMaxRB).
+cudaError_t launch_dabsmax(const AggArgs &a, int B, cudaStream_t st);
+cudaError_t launch_gc_tc(const AggArgs &a, int rb, int B, cudaStream_t st);
 
 }  // namespace sgb

@@ -440,7 +440,7 @@ def test_gradients_at_tile_edges_match_the_oracle(W, H, D, win, bil):
                                        (70, 18, 7, 1), (40, 12, 3, 3), (45, 17, 36, 5), (64, 8, 97, 7), (37, 30, 1, 11),
                                        (3, 40, 30, 13), (50, 21, 34, 15)])
 def test_aggregation_at_strip_and_chunk_edges_matches_the_oracle(W, H, D, bil):
-    """Sizes around the tensor-core form's 32-column strips, 4-row bands, chunks of 32 disparities in
+    """Sizes around the tensor-core adjoint's 32-column strips, 4-row bands, chunks of 32 disparities in
     groups of 4, for every window radius (15 takes the FP32 form); disparity and both gradients by the
     file's bars, and a second backward pass on the same workspace equal to the first."""
     rng = np.random.default_rng(W * 1000 + H * 10 + D)
