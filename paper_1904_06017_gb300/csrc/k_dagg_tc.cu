@@ -14,8 +14,8 @@
 // (the products are exact; w_lo h_lo is below 2^-22).  h comes split from the kernel that writes it
 // (k_diff.cuh: the layout): no conversion on the way into the ring.  Weights are formed in FP32 as in
 // k_dagg and scaled by 2^14; h, which has the range of the caller's dS/dl, by a power of two from the
-// image's largest finite |dS/dl|.  Error of both gradients against 64 bits: below the FP32 form's on five seeds of 8 x 960 x
-// 540 (reference 5.40e-6 -> 5.37e-6, target 4.19e-6 -> 4.07e-6).
+// image's largest finite |dS/dl|.  Error of the gradients against 64 bits: below the FP32 form's on five
+// seeds of 8 x 960 x 540 (reference 5.40e-6 -> 5.37e-6, target 4.19e-6 -> 4.07e-6 on the first).
 //
 // What is not finite, or out of the split's range, is flagged by row where it is written; a patch
 // whose window rows hold a flagged row sums one value at a time instead, so that a NaN reaches the pixels
@@ -29,7 +29,8 @@
 // an FP32 h (2.81 ms), 64 disparities a chunk in one CTA with pairs of warps sharing a patch (3.12), the
 // same without pairs (3.37).  FWD and H in this form (1.73 -> 1.48 and 3.30 -> 2.53 ms) are left out too:
 // their error against 64 bits is lower than the FP32 form's, but where a target window is nearly flat
-// the rounding of E reaches 9e-4 of a gradient's root mean square, so that the two forms differ by as much.
+// the FP32 form's rounding of E reaches 1.3e-3 of a gradient's root mean square, and the two forms
+// differ by as much.
 #include <math.h>
 
 #include "internal.cuh"
