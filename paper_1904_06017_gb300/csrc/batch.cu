@@ -29,6 +29,7 @@ struct stereo_batch {
     };
     std::vector<MarchGroup> march;
     sgb::MarchItem *d_march = nullptr;
+    int ctas = 1;                            // of k_refine per SM
     int ntiles = 0;                          // (pair, tile) items of the whole batch
     size_t smem = 0;
     int nsm = 0;
@@ -167,7 +168,16 @@ static int build(stereo_batch *b, int wc, int dc)
     b->dc = dc;
     const bool sc = wc == kScWC;
     const int rb = b->bp.bil / 2;
-    b->kernel = !sc ? pick_fused(b->bp.cost_dtype, rb, dc, wc) : b->bp.cost_dtype == STEREO_F32 ? pick_refine(rb, false) : nullptr;
+    // k_refine's tiles: by the rule of single frames, over the tiles of all pairs that it works on (36 rows ->
+    // the rule: two pairs, 256 x 192 and 384 x 216, 134 -> 120 us; five, 265 x 199 to 795 x 447, k = 7, 341 ->
+    // 304; six, 288 x 216 to 864 x 486, 459 -> 432)
+    int nref = 0;
+    for (const stereo_ctx *c : b->ctx)
+        if (c->g.D > 32) nref += c->g.ntx * c->g.nty;
+    const int rows = refine_rows(nref, b->nsm);
+    b->ctas = sc ? refine_ctas(nref, b->nsm, rb) : 1;
+    b->kernel = !sc ? pick_fused(b->bp.cost_dtype, rb, dc, wc)
+                : b->bp.cost_dtype == STEREO_F32 ? pick_refine(rb, false, rows, b->ctas) : nullptr;
     if (!fused_available(b->bp.cost_dtype, rb, dc, wc)) {
         release_build(b);
         return set_error(STEREO_ENOTSUP, "batch: no fused kernel for bil=%d dc=%d wc=%d type=%d", b->bp.bil, dc,
@@ -178,7 +188,7 @@ static int build(stereo_batch *b, int wc, int dc)
     b->tile_smem = 0;
     for (stereo_ctx *c : b->ctx) {
         const Geometry &g = c->g;
-        b->smem = std::max(b->smem, sc ? refine_smem_bytes(g) : g.smem_bytes);
+        b->smem = std::max(b->smem, sc ? refine_smem_bytes(g, rows) : g.smem_bytes);
         if (sc) b->tile_smem = std::max(b->tile_smem, sc_smem_bytes(g));
     }
     if (b->kernel && (rc = cuda_error(cudaFuncSetAttribute((const void *)b->kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -211,7 +221,8 @@ static int build(stereo_batch *b, int wc, int dc)
         b->ntiles += g.ntx * g.nty;
         if (sc && b->bp.cost_dtype != STEREO_F32) continue;   // (k_march finishes the 16-bit form itself)
         if (sc && g.D <= 32) b->ntile += g.ntx * g.nty;
-        for (int ty = 0; ty < g.nty; ++ty)
+        const int nty = sc && g.D > 32 ? (g.H + rows - 1) / rows : g.nty;
+        for (int ty = 0; ty < nty; ++ty)
             for (int tx = 0; tx < g.ntx; ++tx) items.push_back({g.Dp, i, tx | (ty << 16)});
     }
     // heaviest tiles first (the work of a tile grows with its pair's search range), after those of
@@ -274,7 +285,7 @@ static int enqueue_fused(stereo_batch *b, cudaStream_t s)
     }
     for (size_t k = 0; k + 1 < ng; ++k) join(k);
     if (rest && !rc) {                      // (none where every pair is done: the 16-bit form, tiles only)
-        const int grid = std::min(b->nsm, rest);
+        const int grid = std::min(b->ctas * b->nsm, rest);
         b->kernel<<<grid, fused_threads(b->wc), b->smem, s>>>(unused, b->d_pairs, b->d_items + b->ntile, rest, b->d_counter);
         rc = cuda_error(cudaGetLastError(), "batch: fused launch");
     }

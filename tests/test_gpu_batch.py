@@ -168,3 +168,31 @@ def test_graph_replay_sees_new_inputs_and_fp16_batch():
     total = sum(a[0].size for a in f)
     diff = sum(int(np.count_nonzero(np.rint(a[0]) != np.rint(b[0]))) for a, b in zip(f, h))
     assert diff / total <= 5e-3
+
+
+@pytest.mark.parametrize("sizes", [[(96, 70, 40)], [(150, 37, 36), (90, 25, 20), (160, 49, 64)],
+                                   [(960, 541, 40), (110, 30, 33)]])
+def test_low_refinement_tiles_equal_single_calls(sizes):
+    """Batches on both sides of the size up to which the refinement's tiles have 12 rows (960 x 541
+    has 480 of 36 rows): equal to the pairs' single calls bit for bit."""
+    qs = []
+    for i, (W, H, D) in enumerate(sizes):
+        rng = np.random.default_rng(W + H + D)
+        ref = rng.integers(0, 256, (H, W), dtype=np.uint8)
+        pitch = pitch_of(W)
+        q = dict(ref=dev_img(ref, pitch), tgt=dev_img(np.roll(ref, -5, axis=1), pitch),
+                 shift=dev_f32((np.arange(H) % 5 - 2).astype(np.float32)),
+                 tgt_warped=torch.zeros((H, pitch), dtype=torch.uint8, device="cuda"), max_disp=D)
+        q.update(disp=torch.zeros((H, W), device="cuda"), disp_out=torch.zeros((H, W), device="cuda"),
+                 valid=torch.zeros((H, W), dtype=torch.uint8, device="cuda"),
+                 res=torch.zeros(64, dtype=torch.uint8, device="cuda"))
+        qs.append(q)
+    with sg.StereoBatch(qs, win=7, bil=9, sigma0=3.0, sigma1=10.0, tile_wc=32, tile_dc=32) as b:
+        b.run()
+        torch.cuda.synchronize()
+        b.check_device_status()
+    for (W, H, D), q in zip(sizes, qs):
+        disp, valid = torch.empty_like(q["disp"]), torch.empty_like(q["valid"])
+        with sg.Stereo(W, H, D, win=7, bil=9, sigma0=3.0, sigma1=10.0, pitch=q["ref"].shape[1]) as st:
+            st.cost_aggregate_wta(q["ref"], q["tgt_warped"], q["shift"], disp, None, valid)
+        assert torch.equal(q["disp"], disp) and torch.equal(q["valid"], valid)
