@@ -1,6 +1,5 @@
 // k_diff.cu -- soft-argmin disparity over the bilateral-aggregated cost and its adjoint
-// (include/stereo_diff.h).  FP32 throughout (but that h goes from H to GC, up to bil = 13, as pairs of FP16
-// halves, 22 bits: k_diff.cuh); the aggregated volume E(p,d) of eq. (fbs) is
+// (include/stereo_diff.h).  FP32 throughout; the aggregated volume E(p,d) of eq. (fbs) is
 // never stored: the backward pass recomputes it tile by tile from the stored cost volume.
 //
 // Forward (per pair of a batch, float images):
@@ -11,13 +10,11 @@
 //   k_dagg<FWD> E(p,d) = sum_q w c / sum_q w (eq. omega_s, eq. fbs), online soft-max over d:
 //               l = sum_d d P(p,d) + s_i(v), P = softmax_d(-E/T); keeps log2-sum-exp, lbar
 // Backward, given gl = dS/dl:
-//   k_dabsmax   the scale of h, from max |gl| of each image
 //   k_dagg<H>   recompute E; gE = -gl P (d - lbar) / T; h = gE / Z(p);  beta(p) = sum_d h E;
 //               t1(p) = sum_d h(p,d) sum_q w (I_q - I_p) c(q,d) - beta(p) sum_q w (I_q - I_p)
-//   agg GC      gc(q,d) = sum_p w(p,q) h(p,d)                  (adjoint of eq. fbs in c)
+//   k_dagg<GC>  gc(q,d) = sum_p w(p,q) h(p,d)                  (adjoint of eq. fbs in c)
 //               gw(x) = 2/sigma1^2 (t1(x) + sum_d c(x,d) sum_q w (I_q - I_x) h(q,d)
 //                                        - sum_q w (I_q - I_x) beta(q))  (through the weights)
-//               (k_dagg_tc.cu up to bil = 13, k_dagg<GC> here at 15)
 //   k_dcost_bwd adjoint of eq. (c).  Per window pair (q, d), with g = gc(q,d) / n and the target
 //               block qt = q - d:  A = -g / (s_a s_b),  B = g ncc / s_a^2,  C = g ncc / s_b^2;
 //               an extended reference position X collects
@@ -40,7 +37,6 @@
 #include <type_traits>
 
 #include "internal.cuh"
-#include "k_diff.cuh"
 #include "row_shift.cuh"
 #include "stereo_diff.h"
 
@@ -48,6 +44,7 @@ namespace sgb {
 namespace {
 
 
+enum { AGG_FWD = 0, AGG_H = 1, AGG_GC = 2 };
 // pixels per thread in k_dagg (a column segment): the forward pass, with one accumulator set,
 // takes 8, so that each staged neighbour row serves twice the weights
 __host__ __device__ constexpr int agg_rows(int mode) { return mode == AGG_FWD ? 8 : 4; }
@@ -107,8 +104,6 @@ struct Dims {
 struct Ws {
     float *tw, *mur, *sdr, *mut, *isdt, *cost, *lse, *lbar;      // forward (isdt: 1 / s_b, 0 where flat)
     float *h, *gc, *beta, *t1, *gw, *gpart, *gqpart, *samb, *sb, *grefx, *gtwx;      // backward
-    unsigned *range;               // split h: its scale, and the rows that the split cannot carry
-    int *hbad;
 };
 
 size_t layout(const Dims &d, char *base, Ws *w)
@@ -118,8 +113,7 @@ size_t layout(const Dims &d, char *base, Ws *w)
         if (p) *p = base ? (float *)(base + off) : nullptr;
         off += (elems * sizeof(float) + 255) / 256 * 256;
     };
-    const size_t B = d.B, img = (size_t)d.H * d.W, vol = (size_t)d.D * img,
-                 volh = (size_t)((d.D + 3) / 4 * 4) * img;   // (h: groups of 4 in the split layout)
+    const size_t B = d.B, img = (size_t)d.H * d.W, vol = (size_t)d.D * img;
     Ws tmp;
     Ws *o = w ? w : &tmp;
     take(&o->tw, B * img);
@@ -133,7 +127,7 @@ size_t layout(const Dims &d, char *base, Ws *w)
     // h, and in its place once it has been read the cost adjoint's sums along q - d
     const size_t gq = (2 * B * (size_t)d.H * cb_tiles_x(d.Wr) * cb_diag_w(d.D) + 63) / 64 * 64, im = (B * img + 63) / 64 * 64;
     const size_t share = gq + 2 * im;
-    take(&o->h, B * volh > share ? B * volh : share);
+    take(&o->h, B * vol > share ? B * vol : share);
     o->gqpart = o->h;
     o->samb = o->h ? o->h + gq : nullptr;
     o->sb = o->h ? o->h + gq + im : nullptr;
@@ -142,8 +136,6 @@ size_t layout(const Dims &d, char *base, Ws *w)
     take(&o->t1, B * img);
     take(&o->gw, B * img);
     take(&o->gpart, B * (size_t)d.Hr * cb_tiles_x(d.Wr) * cb_diag_w(d.D));
-    take((float **)&o->range, B * kAggRange);
-    take((float **)&o->hbad, B * (size_t)d.H);
     take(&o->grefx, B * (size_t)d.Hr * d.Wr);
     take(&o->gtwx, B * (size_t)d.Hr * d.Wt);
     return off;
@@ -464,6 +456,27 @@ __global__ void __launch_bounds__(kCostThreads, 3) k_dcost(const float *__restri
 }
 
 // ------------------------------------------------------------------ aggregation stencil
+struct AggArgs {
+    const float *img;      // reference image [B][H][W]
+    const float *vol;      // neighbour values [B][D][H][W]: the cost (FWD, H) or h (GC)
+    const float *shift;    // FWD: row shifts
+    float *disp;           // FWD: l
+    float *lse, *lbar;     // FWD out, H in
+    const float *gdisp;    // H: dS/dl
+    float *h;              // H out
+    float *beta, *t1;      // H out, GC in
+    float *gc;             // GC out
+    const float *cost;     // GC: c(x, d) of the centre pixel
+    float *gw;             // GC out: image gradient through the weights
+    int W, H, D;
+    int warp_mode;         // FWD: the add-back is s_i (rounded) or s(v) (linear warp)
+    float kappa;           // sqrt(log2 e) / sigma1: scaled intensities
+    float k0;              // -log2 e / sigma0^2
+    float kT;              // log2 e / T
+    float invT;            // 1 / T
+    float gw_scale;        // 2 / (sigma1^2 kappa)
+};
+
 // The disparity chunks of a tile are staged in two shared-memory buffers: while chunk k is
 // aggregated, the copies of chunk k + 1 are in flight (cp.async, 4 bytes per element, zero
 // fill outside the image and beyond D).
@@ -492,7 +505,6 @@ __global__ void __launch_bounds__(agg_threads(MODE), MODE == AGG_FWD ? 3 : MODE 
     constexpr int kAggTX = agg_tx(MODE), kAggTY = agg_ty(MODE), kAggThreads = agg_threads(MODE);
     constexpr int TW = kAggTX + 2 * RB, TH = kAggTY + 2 * RB;
     constexpr bool TWO = MODE != AGG_FWD;
-    constexpr bool SPLIT = MODE == AGG_H && RB <= kAggTcMaxRB;     // h goes to k_dagg_tc
     extern __shared__ float4 smem4[];
     float4 *Vbuf = smem4;                                     // [1 or 2][NQ][TH][TW]
     float *sI = (float *)(Vbuf + (DB ? 2 : 1) * NQ * TH * TW); // [TH][TW]
@@ -548,8 +560,6 @@ __global__ void __launch_bounds__(agg_threads(MODE), MODE == AGG_FWD ? 3 : MODE 
             if (i < TH * TW) sI[i] = vi[it];
         }
     }
-    float hscale = 1.f;
-    if constexpr (SPLIT) hscale = pow2i(h_shift(a, b, threadIdx.x & 31));
     float ky[2 * RB + 1];
 #pragma unroll
     for (int j = 0; j <= 2 * RB; ++j) ky[j] = a.k0 * (float)((j - RB) * (j - RB));
@@ -691,36 +701,16 @@ __global__ void __launch_bounds__(agg_threads(MODE), MODE == AGG_FWD ? 3 : MODE 
                 st1[i] = s0;
                 st2[i] = s1;
             } else if constexpr (MODE == AGG_H) {
-                float hk[DC];
 #pragma unroll
                 for (int k = 0; k < DC; ++k) {
                     const int d = d0 + k;
-                    hk[k] = 0.f;
-                    if (d >= D) continue;
+                    if (d >= D) break;
                     const float E = lane(acc0[i][k >> 1], k) * invZ[i];
                     const float P = exp2f(-E * a.kT - st1[i]);
                     const float hv = -st0[i] * a.invT * P * ((float)d - st2[i]) * invZ[i];
-                    if constexpr (!SPLIT) a.h[((size_t)b * D + d) * HW + pix] = hv;
-                    hk[k] = hv;
+                    a.h[((size_t)b * D + d) * HW + pix] = hv;
                     beta[i] = fmaf(hv, E, beta[i]);
                     tacc[i] = fmaf(hv, lane(acc1[i][k >> 1], k), tacc[i]);
-                }
-                if constexpr (SPLIT) {
-                    bool off = false;
-#pragma unroll
-                    for (int q = 0; q < DC / 4; ++q) {
-                        if (d0 + 4 * q >= D) break;
-                        uint4 v;
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            hk[4 * q + k] *= hscale;
-                            off |= off_range(hk[4 * q + k]);
-                        }
-                        split2(hk[4 * q], hk[4 * q + 1], v.x, v.z);
-                        split2(hk[4 * q + 2], hk[4 * q + 3], v.y, v.w);
-                        reinterpret_cast<uint4 *>(a.h)[((size_t)b * ((D + 3) / 4) + d0 / 4 + q) * HW + pix] = v;
-                    }
-                    if (off) a.hbad[b * H + py[i]] = 1;
                 }
             } else {
 #pragma unroll
@@ -1316,20 +1306,16 @@ cudaError_t launch_agg_rb(const AggArgs &a, int B, cudaStream_t st)
 template <int MODE>
 cudaError_t launch_agg(const AggArgs &a, int rb, int B, cudaStream_t st)
 {
-    if constexpr (MODE != AGG_GC) {
-        switch (rb) {
-        case 0: return launch_agg_rb<MODE, 0>(a, B, st);
-        case 1: return launch_agg_rb<MODE, 1>(a, B, st);
-        case 2: return launch_agg_rb<MODE, 2>(a, B, st);
-        case 3: return launch_agg_rb<MODE, 3>(a, B, st);
-        case 4: return launch_agg_rb<MODE, 4>(a, B, st);
-        case 5: return launch_agg_rb<MODE, 5>(a, B, st);
-        case 6: return launch_agg_rb<MODE, 6>(a, B, st);
-        }
-    } else if (rb <= kAggTcMaxRB) {       // (k_dagg_tc.cu has both sides' times)
-        return launch_gc_tc(a, rb, B, st);
+    switch (rb) {
+    case 0: return launch_agg_rb<MODE, 0>(a, B, st);
+    case 1: return launch_agg_rb<MODE, 1>(a, B, st);
+    case 2: return launch_agg_rb<MODE, 2>(a, B, st);
+    case 3: return launch_agg_rb<MODE, 3>(a, B, st);
+    case 4: return launch_agg_rb<MODE, 4>(a, B, st);
+    case 5: return launch_agg_rb<MODE, 5>(a, B, st);
+    case 6: return launch_agg_rb<MODE, 6>(a, B, st);
+    default: return launch_agg_rb<MODE, 7>(a, B, st);
     }
-    return launch_agg_rb<MODE, kAggTcMaxRB + 1>(a, B, st);
 }
 
 template <int RW>
@@ -1472,10 +1458,7 @@ extern "C" int stereo_softargmin_bwd(const stereo_diff_params *p, const float *r
     a.h = w.h;
     a.beta = w.beta;
     a.t1 = w.t1;
-    a.range = w.range;
-    a.hbad = w.hbad;
-    cudaError_t e = d.rb <= kAggTcMaxRB ? launch_dabsmax(a, B, st) : cudaSuccess;
-    if (e == cudaSuccess) e = launch_agg<AGG_H>(a, d.rb, B, st);
+    cudaError_t e = launch_agg<AGG_H>(a, d.rb, B, st);
     if (e != cudaSuccess) return cuda_error(e, who);
     a.vol = w.h;
     a.gc = w.gc;

@@ -487,3 +487,26 @@ def test_what_is_not_finite_stays_in_its_windows(bil):
     r = rb + rw + 32
     assert np.isnan(gr[0, y, x]) and np.isfinite(gr[0][(abs(v - y) > r) | (abs(u - x) > r)]).all()
     assert np.isfinite(gt[0][(abs(v - y) > r) | (u > x + r) | (u < x - r - D + 1)]).all()
+
+
+@pytest.mark.parametrize("bil", [5, 11, 13, 15])
+@pytest.mark.parametrize("r,kind", [(1e-4, "half"), (1e-6, "half"), (1e-8, "half"), (1e-12, "half"), (1e-9, "pixel")])
+def test_gradients_hold_where_dl_is_far_below_the_largest(bil, r, kind):
+    """dS/dl of one part of the image a fraction r of the other's (the top half's, or one pixel's): the
+    gradients of the small part, beyond both windows and a tile of the cost adjoint, by the file's bar
+    of their own largest value."""
+    W, H, D, win = 48, 128, 20, 5
+    rng = np.random.default_rng(bil)
+    ref, tgt = rng.uniform(0, 255, (H, W)), rng.uniform(0, 255, (H, W))
+    sh = rng.uniform(-3, 6, H).astype(np.float32)
+    gl = rng.normal(size=(H, W)).astype(np.float32)
+    if kind == "half":
+        gl[48:] *= np.float32(r)
+    else:
+        gl[47, 24] /= np.float32(r)
+    l, p, rts, ws = gpu_forward([ref], [tgt], [sh], D, win, bil)
+    _, gro, gto = odiff.disparity_vjp(ref, tgt, sh, D, win, bil, S0, S1, T, gl.astype(np.float64))
+    gr, gt = gpu_backward(p, rts, ws, gl[None])
+    y = 48 + bil // 2 + win // 2 + 24 + win - 1
+    check_grad(gr[0][y:], gro[y:], "dS/dref")
+    check_grad(gt[0][y:], gto[y:], "dS/dtgt")
