@@ -176,7 +176,9 @@ int launch_cost_volume(stereo_ctx *ctx, float *cost, cudaStream_t s)
 // through L1 instead.  640 x 360, D = 32, k = 11: 93 us, 19 TFLOP/s (2.95 ms).
 constexpr int kAvDC = 16, kAvTX = 32, kAvTY = 16, kAvPY = 4;
 constexpr int kAvThreads = 32 * kAvTY / kAvPY;
-constexpr float kAvFar = 1e18f;    // intensity of an out-of-image neighbour: weight 0
+// Intensity of an out-of-image neighbour: its exponent is -infinity for every 1 / sigma1^2 > 0, so its
+// weight is 0 (the intensities are staged unscaled: a finite value would count once sigma1 is as large).
+constexpr float kAvFar = INFINITY;
 
 template <int RB>
 __global__ void __launch_bounds__(kAvThreads)
@@ -287,7 +289,9 @@ int launch_aggregate_volume(stereo_ctx *ctx, const uint8_t *ref, const float *co
 {
     const Geometry &g = ctx->g;
     const float s0 = ctx->p.sigma0, s1 = ctx->p.sigma1;
-    const float i0 = 1.0f / (s0 * s0), i1 = 1.0f / (s1 * s1);
+    // (1 / sigma1^2 at least the smallest positive float, which leaves every weight of two pixels as it
+    // is and keeps the exponent of an out-of-image neighbour from becoming 0 x infinity)
+    const float i0 = 1.0f / (s0 * s0), i1 = fmaxf(1.0f / (s1 * s1), 0x1p-149f);
     const int vec = g.D % 4 == 0 && (((uintptr_t)cost | (uintptr_t)agg) & 15) == 0;
     cudaError_t e;
     switch (g.rb) {

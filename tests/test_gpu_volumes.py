@@ -77,3 +77,17 @@ def test_wta_volume_scan(D):
     b2 = best2.cpu().numpy()
     assert np.array_equal(b2[..., 0], np.take_along_axis(e, best[..., None], 2)[..., 0], equal_nan=True)
     assert np.array_equal(b2[..., 1], second)
+
+
+@pytest.mark.parametrize("sigma1", [1e16, 1e17, 1e18, 1e19, 1e25, 3e38])
+def test_aggregation_without_a_range_term(sigma1):
+    """A sigma1 so large that intensities don't matter: at the borders too, only the neighbours inside
+    the image count."""
+    W, H, D, bil = 37, 21, 9, 11
+    rng = np.random.default_rng(5)
+    ref = synth.texture(rng, H, W)
+    cost = rng.uniform(0, 2, (H, W, D)).astype(np.float32)
+    agg = torch.empty((H, W, D), device="cuda")
+    with sg.Stereo(W, H, D, win=3, bil=bil, sigma0=3.0, sigma1=sigma1, pitch=pitch_of(W)) as st:
+        st.aggregate_volume(dev_img(ref, pitch_of(W)), dev_f32(cost), agg)
+    check_rel(agg.cpu().numpy(), oracle.aggregate(ref, cost, bil, 3.0, sigma1))
