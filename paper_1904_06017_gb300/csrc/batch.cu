@@ -135,9 +135,7 @@ static int build_march(stereo_batch *b)
         std::stable_sort(best.begin(), best.end(), [&](const MarchItem &x, const MarchItem &y) { return cost(x) > cost(y); });
         const Geometry &g = b->ctx[best[0].pair]->g;
         const MarchChoice c = pick_march(b->bp.cost_dtype, g.rb, g.rw, g.D);
-        const int rc = cuda_error(cudaFuncSetAttribute((const void *)c.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                       (int)c.smem),
-                                  "batch: cudaFuncSetAttribute");
+        const int rc = allow_smem((const void *)c.kernel, c.smem, "batch: cudaFuncSetAttribute");
         if (rc) return rc;
         b->march.push_back({c, (int)all.size(), (int)best.size()});
         all.insert(all.end(), best.begin(), best.end());
@@ -191,9 +189,7 @@ static int build(stereo_batch *b, int wc, int dc)
         b->smem = std::max(b->smem, sc ? refine_smem_bytes(g, rows) : g.smem_bytes);
         if (sc) b->tile_smem = std::max(b->tile_smem, sc_smem_bytes(g));
     }
-    if (b->kernel && (rc = cuda_error(cudaFuncSetAttribute((const void *)b->kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                           (int)b->smem),
-                                      "batch: cudaFuncSetAttribute"))) {
+    if (b->kernel && (rc = allow_smem((const void *)b->kernel, b->smem, "batch: cudaFuncSetAttribute"))) {
         release_build(b);
         return rc;
     }
@@ -203,9 +199,7 @@ static int build(stereo_batch *b, int wc, int dc)
     }
     b->ntiles = 0;
     if (b->kernel && sc &&
-        (rc = cuda_error(cudaFuncSetAttribute((const void *)pick_fused_sc(rb), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)b->tile_smem),
-                         "batch: cudaFuncSetAttribute"))) {
+        (rc = allow_smem((const void *)pick_fused_sc(rb), b->tile_smem, "batch: cudaFuncSetAttribute"))) {
         release_build(b);
         return rc;
     }

@@ -187,6 +187,10 @@ int compute_geometry(const stereo_params &p, int dc, int wc, Geometry &g);
 // Context creation with a given (disparities per chunk, warp columns); 0 = default choice.
 int create_context(const stereo_params *p, int dc, int wc, stereo_ctx **out);
 int max_smem_optin();
+// Lets a kernel be launched with `bytes` of dynamic shared memory.  The limit is one value per kernel and
+// device, for every context, batch and thread: it is set to all that the device allows beside the kernel's
+// static part, so that no later call lowers it under a context that needs more.
+int allow_smem(const void *kernel, size_t bytes, const char *what);
 int launch_cost_volume(stereo_ctx *ctx, float *cost, cudaStream_t s);
 int launch_aggregate_volume(stereo_ctx *ctx, const uint8_t *ref, const float *cost, float *agg,
                             cudaStream_t s);

@@ -1322,8 +1322,9 @@ template <int RW>
 cudaError_t launch_cb_rw(const CbArgs &a, int B, cudaStream_t st)
 {
     const size_t smem = CbShape<RW>::smem(a.D);
+    // (the same limit in every call, that of the longest range: another thread's call must not lower it)
     cudaError_t e = cudaFuncSetAttribute(k_dcost_bwd<RW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+                                         (int)CbShape<RW>::smem(kMaxD));
     if (e != cudaSuccess) return e;
     dim3 grid((a.Wr + 31) / 32, (a.Hr + CbShape<RW>::TY - 1) / CbShape<RW>::TY, B);
     k_dcost_bwd<RW><<<grid, 256, smem, st>>>(a);

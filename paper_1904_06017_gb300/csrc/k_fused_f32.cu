@@ -63,11 +63,6 @@ static FusedKernel pick(const stereo_ctx *ctx)
     return pick_fused(ctx->p.cost_dtype, ctx->g.rb, ctx->g.dc, ctx->g.wc);
 }
 
-static int set_smem(const void *k, size_t bytes, const char *what)
-{
-    return cuda_error(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes), what);
-}
-
 int fused_configure(stereo_ctx *ctx)
 {
     const Geometry &g = ctx->g;
@@ -77,38 +72,33 @@ int fused_configure(stereo_ctx *ctx)
         const bool f32 = ctx->p.cost_dtype == STEREO_F32;
         int rc;
         if (f32 && sc_route(g.W, g.H, g.D) == kRouteTile) {
-            rc = set_smem((const void *)pick_fused_sc(g.rb), sc_smem_bytes(g), "cudaFuncSetAttribute(tiles)");
+            rc = allow_smem((const void *)pick_fused_sc(g.rb), sc_smem_bytes(g), "cudaFuncSetAttribute(tiles)");
         } else {
             const MarchChoice c = pick_march(ctx->p.cost_dtype, g.rb, g.rw, g.D);
-            rc = set_smem((const void *)c.kernel, c.smem, "cudaFuncSetAttribute(march)");
+            rc = allow_smem((const void *)c.kernel, c.smem, "cudaFuncSetAttribute(march)");
             if (!rc && march_split(g.rb, g.D)) {
                 const MarchChoice m = pick_march(ctx->p.cost_dtype, g.rb, g.rw, march_split(g.rb, g.D)),
                                   r = pick_march_rest(ctx->p.cost_dtype, g.rb, g.rw, g.D);
-                rc = set_smem((const void *)m.kernel, m.smem, "cudaFuncSetAttribute(march)");
-                if (!rc) rc = set_smem((const void *)r.kernel, r.smem, "cudaFuncSetAttribute(march)");
+                rc = allow_smem((const void *)m.kernel, m.smem, "cudaFuncSetAttribute(march)");
+                if (!rc) rc = allow_smem((const void *)r.kernel, r.smem, "cudaFuncSetAttribute(march)");
             }
         }
         if (rc || !f32) return rc;
         const size_t rs = refine_smem_bytes(g);
         for (int ctas = 1; ctas <= 2; ++ctas)
-            if ((rc = set_smem((const void *)pick_refine(g.rb, false, kRefineRows, ctas), refine_smem_bytes(g, kRefineRows),
-                               "cudaFuncSetAttribute(refine)")))
+            if ((rc = allow_smem((const void *)pick_refine(g.rb, false, kRefineRows, ctas), refine_smem_bytes(g, kRefineRows),
+                                 "cudaFuncSetAttribute(refine)")))
                 return rc;
-        if ((rc = set_smem((const void *)pick_refine(g.rb, false), rs, "cudaFuncSetAttribute(refine)"))) return rc;
-        return set_smem((const void *)pick_refine(g.rb, true), rs, "cudaFuncSetAttribute(refine, best2)");
+        if ((rc = allow_smem((const void *)pick_refine(g.rb, false), rs, "cudaFuncSetAttribute(refine)"))) return rc;
+        return allow_smem((const void *)pick_refine(g.rb, true), rs, "cudaFuncSetAttribute(refine, best2)");
     }
     FusedKernel k = pick(ctx);
     if (!k)
         return set_error(STEREO_ENOTSUP, "no fused kernel for bil=%d dc=%d cost_dtype=%d", ctx->p.bil, ctx->g.dc,
                          ctx->p.cost_dtype);
-    int rc = cuda_error(cudaFuncSetAttribute((const void *)k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)ctx->g.smem_bytes),
-                        "cudaFuncSetAttribute(fused)");
+    int rc = allow_smem((const void *)k, ctx->g.smem_bytes, "cudaFuncSetAttribute(fused)");
     FusedKernel k2 = pick_fused_b2(ctx->p.cost_dtype, ctx->g.rb, ctx->g.dc, ctx->g.wc);
-    if (!rc && k2)
-        rc = cuda_error(cudaFuncSetAttribute((const void *)k2, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)ctx->g.smem_bytes),
-                        "cudaFuncSetAttribute(fused, best2)");
+    if (!rc && k2) rc = allow_smem((const void *)k2, ctx->g.smem_bytes, "cudaFuncSetAttribute(fused, best2)");
     return rc;
 }
 

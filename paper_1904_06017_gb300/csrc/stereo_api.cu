@@ -181,6 +181,16 @@ int max_smem_optin()
     return v;
 }
 
+int allow_smem(const void *kernel, size_t bytes, const char *what)
+{
+    cudaFuncAttributes a;
+    const int rc = cuda_error(cudaFuncGetAttributes(&a, kernel), what);
+    if (rc) return rc;
+    const size_t most = (size_t)max_smem_optin() - a.sharedSizeBytes;
+    return cuda_error(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)(bytes > most ? bytes : most)), what);
+}
+
 // Static shared memory of the fused kernel (pair arguments, work item) on top of the dynamic part.
 constexpr int kFusedStaticSmem = 2048;
 

@@ -99,3 +99,47 @@ def test_refinement_tile_heights_equal_simt(W, H, D, win, bil):
     shift = (np.arange(H) % 5 - 2).astype(np.float32)
     assert_same(run(ref, tgt, shift, D, win, bil, 3.0, 10.0, sg.STEREO_FUSED_SIMT),
                 run(ref, tgt, shift, D, win, bil, 3.0, 10.0, sg.STEREO_FUSED_TENSOR))
+
+
+@pytest.mark.parametrize("form", ["f32", "simt", "f16", "tiles", "small", "batch"])
+def test_context_runs_after_others_of_smaller_windows_and_ranges(form):
+    """A context whose kernels need much shared memory, then contexts that need less of the same kernels
+    (other windows and ranges, a warp estimator, a batch): the first one runs as before."""
+    W, H, D = (400, 300, 30) if form == "tiles" else (200, 80, 30) if form == "small" else (200, 80, 128)
+    ref, tgt, shift = pair(W, H, 5, 3)
+    pitch = pitch_of(W)
+    args = dict(ref=dev_img(ref, pitch), tgt=dev_img(tgt, pitch), shift=dev_f32(shift))
+    disp, wta = torch.empty((H, W), device="cuda"), torch.empty((H, W), dtype=torch.int32, device="cuda")
+    valid = torch.empty((H, W), dtype=torch.uint8, device="cuda")
+
+    def batch(D, win):
+        q = dict(args, max_disp=D, disp=torch.empty((H, W), device="cuda"), disp_out=disp, valid=valid,
+                 tgt_warped=torch.zeros((H, pitch), dtype=torch.uint8, device="cuda"),
+                 res=torch.zeros(64, dtype=torch.uint8, device="cuda"))
+        return sg.StereoBatch([q], win=win, bil=11, sigma0=3.0, sigma1=10.0, tile_wc=32, tile_dc=32), q
+
+    def frame(win, D, **kw):
+        return sg.Stereo(W, H, D, win=win, bil=11, sigma0=3.0, sigma1=10.0, pitch=pitch, **kw)
+
+    kw = dict(simt=dict(fused_form=sg.STEREO_FUSED_SIMT), f16=dict(cost_dtype=sg.STEREO_F16)).get(form, {})
+    if form == "batch":
+        b, q = batch(D, 11)
+
+        def run_it():
+            q["disp"].fill_(-1)
+            b.run()
+            torch.cuda.synchronize()
+            return q["disp"].clone()
+    else:
+        st = frame(11, D, **kw)
+
+        def run_it():
+            disp.fill_(-1)
+            st.cost_aggregate_wta(args["ref"], args["tgt"], args["shift"], disp, wta, valid)
+            torch.cuda.synchronize()
+            return disp.clone()
+    before = run_it()
+    others = [frame(3, d, **k) for d in (100, 40, 5) for k in (kw, {})]
+    others += [sg.WarpEstimator(W, H, 64, factor=2, win=3, bil=11, pitch=pitch), batch(100, 3)[0], batch(5, 3)[0]]
+    assert torch.equal(run_it(), before)
+    del others
