@@ -9,12 +9,13 @@
 //
 // An FP64 instruction of a warp occupies a GB300 SM about 16 times as long as an FP32 one and
 // returns after about 65 cycles, so the per-pixel sums are kept out of FP64: a warp adds its
-// pixels in pairs of floats (the rounding error of every addition and product is recovered
-// exactly and summed beside it, so a sum carries about 48 bits over the thousand or so pixels
-// of a warp) and widens once at the end; sums over pixel coordinates are exact integers.
-// A warp whose pair is not finite (an infinite or NaN disparity, or a sum beyond the FP32
-// range) adds its pixels again in FP64.  8 maps of 960 x 540: energy 13 us (24 us with FP64
-// sums and butterflies), adjoint 18 us (63), moments 22 us (152); all are bound by the FP64
+// pixels in three floats each (the rounding error of every addition and product is recovered
+// exactly and summed in the second, that sum's own in the third, so that a sum carries more than
+// 64 bits) and widens once at the end; sums over pixel coordinates are exact integers.
+// (Two floats, 24 bits for the sum of the errors, left 3e-14 of sum l^2 on a constant map, 200 times
+// the error of FP64 sums.)  A warp whose sum is not finite (an infinite or NaN disparity, or a sum
+// beyond the FP32 range), or whose products leave errors below that range, adds its pixels again in FP64.  8 maps of 960 x 540: energy 15 us (24 us with FP64
+// sums and butterflies), adjoint 23 us (63), moments 32 us (152); all are bound by the FP64
 // tail of a block (the widened warp sums) more than by reading the map.
 #include <cuda_runtime.h>
 #include <math.h>
@@ -39,31 +40,38 @@ size_t dte_bytes(int B)
     return (part + 255) / 256 * 256;
 }
 
-// A sum of floats with the rounding errors of its additions beside it.
-struct PairSum {
-    float hi, lo;
-    __device__ __forceinline__ void add(float x)
-    {
-        const float s = __fadd_rn(hi, x), b = __fsub_rn(s, hi);
-        lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(x, b)));
-        hi = s;
-    }
-    // += the exact product x y
+// s + x, and what its rounding leaves.
+__device__ __forceinline__ float two_sum(float &s, float x)
+{
+    const float t = __fadd_rn(s, x), b = __fsub_rn(t, s), e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(x, b));
+    s = t;
+    return e;
+}
+
+// A sum of floats: hi, the rounding errors of its additions in mid, and those of mid's in lo.
+struct TripleSum {
+    float hi, mid, lo;
+    __device__ __forceinline__ void add_error(float x) { lo = __fadd_rn(lo, two_sum(mid, x)); }
+    __device__ __forceinline__ void add(float x) { add_error(two_sum(hi, x)); }
+    // += the exact product x y (its error is exact unless it falls below the FP32 range)
     __device__ __forceinline__ void add_product(float x, float y)
     {
         const float p = __fmul_rn(x, y);
-        lo = __fadd_rn(lo, __fmaf_rn(x, y, -p));
+        add_error(__fmaf_rn(x, y, -p));
         add(p);
     }
-    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
-    // the total over the 32 lanes of a warp, on every lane
+    __device__ __forceinline__ bool finite() const { return isfinite(hi) && isfinite(mid) && isfinite(lo); }
+    __device__ __forceinline__ double value() const { return (double)hi + ((double)mid + (double)lo); }
+    // the total over the 32 lanes of a warp, the same bits on every lane (each step is symmetric in the
+    // two lanes that meet)
     __device__ __forceinline__ void warp_add()
     {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
-            const float h = __shfl_xor_sync(0xffffffffu, hi, o), l = __shfl_xor_sync(0xffffffffu, lo, o);
-            add(h);
-            lo = __fadd_rn(lo, l);
+            const float h = __shfl_xor_sync(0xffffffffu, hi, o), m = __shfl_xor_sync(0xffffffffu, mid, o),
+                        l = __shfl_xor_sync(0xffffffffu, lo, o);
+            const float eh = two_sum(hi, h), em = two_sum(mid, m), ee = two_sum(mid, eh);
+            lo = __fadd_rn(__fadd_rn(lo, l), __fadd_rn(em, ee));
         }
     }
 };
@@ -143,9 +151,9 @@ __global__ void __launch_bounds__(kDteThreads) k_dte(const float *__restrict__ d
     };
     constexpr int kStep = kDteBlocks * kDteThreads, kAhead = 4;   // loads in flight per thread
     const int i0 = blockIdx.x * kDteThreads + threadIdx.x;
-    PairSum ps[NS];
+    TripleSum ps[NS];
 #pragma unroll
-    for (int k = 0; k < NS; ++k) ps[k] = PairSum{0.f, 0.f};
+    for (int k = 0; k < NS; ++k) ps[k] = TripleSum{0.f, 0.f, 0.f};
     for (int i = i0; i < HW; i += kAhead * kStep) {
         float l[kAhead];
         bool in[kAhead];
@@ -170,10 +178,10 @@ __global__ void __launch_bounds__(kDteThreads) k_dte(const float *__restrict__ d
 #pragma unroll
     for (int k = 0; k < NS; ++k) {
         ps[k].warp_add();
-        finite = finite && isfinite(ps[k].hi) && isfinite(ps[k].lo);
+        finite = finite && ps[k].finite();
         acc[k] = ps[k].value();
     }
-    if (!finite) {   // (the same on every lane)
+    if (!__all_sync(0xffffffffu, finite)) {
 #pragma unroll
         for (int k = 0; k < NS; ++k) acc[k] = 0.0;
         for (int i = i0; i < HW; i += kStep) {
@@ -226,7 +234,7 @@ __global__ void __launch_bounds__(32) k_dte_finish(const double *__restrict__ pa
 // The ten moments of the fitted pixels in coordinates centred on the image:
 // n, S_u, S_v, S_l, S_uu, S_uv, S_vv, S_ul, S_vl, S_ll with u' = u - (W-1)/2, v' = v - (H-1)/2.
 // Every sum the refinement needs at an angle psi is a fixed combination of them.  The
-// coordinates enter doubled (whole numbers); the sums with l are pair sums of exact products.
+// coordinates enter doubled (whole numbers); the sums with l are those of exact products.
 __global__ void __launch_bounds__(kDteThreads) k_dref_moments(const float *__restrict__ disp,
                                                               const uint8_t *__restrict__ mask,
                                                               double *__restrict__ part, int W, int H)
@@ -239,7 +247,8 @@ __global__ void __launch_bounds__(kDteThreads) k_dref_moments(const float *__res
     const int i0 = blockIdx.x * kDteThreads + threadIdx.x;
     int n = 0;
     long long su = 0, sv = 0, suu = 0, suv = 0, svv = 0;   // sums over 2u', 2v' and their products
-    PairSum sl{0.f, 0.f}, sul{0.f, 0.f}, svl{0.f, 0.f}, sll{0.f, 0.f};
+    TripleSum sl{0.f, 0.f, 0.f}, sul{0.f, 0.f, 0.f}, svl{0.f, 0.f, 0.f}, sll{0.f, 0.f, 0.f};
+    bool any = false;   // a disparity other than 0
     for (int i = i0; i < HW; i += kAhead * kStep) {
         float l[kAhead];
         bool in[kAhead];
@@ -255,6 +264,7 @@ __global__ void __launch_bounds__(kDteThreads) k_dref_moments(const float *__res
             const int p = i + j * kStep, v = p / W, u = p - v * W;
             const int x = 2 * u - (W - 1), y = 2 * v - (H - 1);
             ++n;
+            any = any || l[j] != 0.f;
             su += x;
             sv += y;
             suu += (long long)x * x;
@@ -274,7 +284,9 @@ __global__ void __launch_bounds__(kDteThreads) k_dref_moments(const float *__res
     double acc[kDteSums] = {(double)n, 0.5 * (double)warp_add(su), 0.5 * (double)warp_add(sv), sl.value(),
                             0.25 * (double)warp_add(suu), 0.25 * (double)warp_add(suv), 0.25 * (double)warp_add(svv),
                             sul.value(), svl.value(), sll.value()};
-    if (!(isfinite(acc[3]) && isfinite(acc[7]) && isfinite(acc[8]) && isfinite(acc[9]))) {   // (the same on every lane)
+    // below 2^-80 the errors of the products l^2 (and with them those of u l, v l) may have underflowed
+    const bool small = __any_sync(0xffffffffu, any) && !(acc[9] >= 0x1p-80);
+    if (__any_sync(0xffffffffu, small || !(sl.finite() && sul.finite() && svl.finite() && sll.finite()))) {
         double f[4] = {0.0, 0.0, 0.0, 0.0};
         for (int i = i0; i < HW; i += kStep) {
             if (M && !M[i]) continue;

@@ -510,3 +510,15 @@ def test_gradients_hold_where_dl_is_far_below_the_largest(bil, r, kind):
     y = 48 + bil // 2 + win // 2 + 24 + win - 1
     check_grad(gr[0][y:], gro[y:], "dS/dref")
     check_grad(gt[0][y:], gto[y:], "dS/dtgt")
+
+
+@pytest.mark.parametrize("H,W,value", [(540, 960, 93.7123), (100, 333, 0.1), (64, 64, 1e-25), (64, 64, 3e18)])
+def test_refinement_sums_carry_64_bits(H, W, value):
+    """A constant map: E = n (C_ll - ...) is the difference of two equal numbers, so it shows the error
+    of sum l^2 and of (sum l)^2 / n.  Each is a chain of at most 15 FP64 additions over a warp's total
+    (2 + 7 + 6), the square takes the second twice: 64 roundings of 2^-53 of n l^2 bound |E|.  alpha0 takes
+    the mean and a slope of as many roundings of E|y| l / C_yy over an image's side."""
+    v = float(np.float32(value))
+    traj = sgd.refine_roll(torch.full((1, H, W), value, device="cuda"), None, 0.3, 2).cpu().numpy()[0]
+    assert np.abs(traj[:, 4]).max() <= 64 * 2.0 ** -53 * H * W * v * v
+    assert np.abs(traj[:, 1] - v).max() <= 64 * (1 + 1.5 * (max(H, W) / min(H, W)) ** 2) * 2.0 ** -53 * v
