@@ -14,9 +14,10 @@
 // 64 bits) and widens once at the end; sums over pixel coordinates are exact integers.
 // (Two floats, 24 bits for the sum of the errors, left 3e-14 of sum l^2 on a constant map, 200 times
 // the error of FP64 sums.)  A warp whose sum is not finite (an infinite or NaN disparity, or a sum
-// beyond the FP32 range), or whose products leave errors below that range, adds its pixels again in FP64.  8 maps of 960 x 540: energy 15 us (24 us with FP64
-// sums and butterflies), adjoint 23 us (63), moments 32 us (152); all are bound by the FP64
-// tail of a block (the widened warp sums) more than by reading the map.
+// beyond the FP32 range), or whose products leave errors below that range, adds its pixels again in
+// FP64.  8 maps of 960 x 540: energy 15 us (24 us with FP64 sums and butterflies), adjoint 23 us
+// (63), moments 32 us (152); bound by the FP64 tail of a block (the widened warp sums) and the
+// two-sums more than by reading the map.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -322,10 +323,10 @@ __device__ double wrap_half_pi_d(double psi)
 //
 // The steps are one FP64 dependency chain, so only what the next angle needs is on it: with
 // C_xx C_yy - C_xy^2 = det, the same at every angle, g / H = C_yy (C_xl C_yy - C_yl C_xy) /
-// (C_yl det), one quotient.  Its reciprocal is an FP32 one with one Newton step in FP64 (about
-// 47 bits: an error of 1e-14 of the step, which the next step corrects), or the full division
-// where FP32 cannot hold the divisor.  The angles go to shared memory, and the trajectory's
-// entries are then evaluated with one step per lane.  50 steps: 102 us (289 us with the sums
+// (C_yl det), one quotient: an FP32 reciprocal with one Newton step in FP64 (about 47 bits), then the
+// quotient corrected by its own remainder (a rounding off; 7e-15 of the step without it), or the
+// full division where FP32 cannot hold the divisor.  The angles go to shared memory, and the trajectory's
+// entries are then evaluated with one step per lane.  50 steps: 106 us (289 us with the sums
 // over raw coordinates and every quantity of a step evaluated on the chain).
 constexpr int kDrefSteps = 1000;   // the most steps a call may ask for
 
@@ -355,8 +356,9 @@ __global__ void __launch_bounds__(32) k_dref_run(const double *__restrict__ part
         const float r0 = 1.0f / (float)den;
         double d;
         if (fabsf(r0) > 1e-30f && fabsf(r0) < 1e30f) {
-            const double r = (double)r0;
-            d = num * (r * (2.0 - den * r));
+            const double r = (double)r0, r1 = r * (2.0 - den * r);
+            d = num * r1;
+            d = fma(fma(-d, den, num), r1, d);
         } else {
             d = num / den;
         }

@@ -522,3 +522,24 @@ def test_refinement_sums_carry_64_bits(H, W, value):
     traj = sgd.refine_roll(torch.full((1, H, W), value, device="cuda"), None, 0.3, 2).cpu().numpy()[0]
     assert np.abs(traj[:, 4]).max() <= 64 * 2.0 ** -53 * H * W * v * v
     assert np.abs(traj[:, 1] - v).max() <= 64 * (1 + 1.5 * (max(H, W) / min(H, W)) ** 2) * 2.0 ** -53 * v
+
+
+@pytest.mark.parametrize("psi", [-0.54, 1.2225, -0.465, 1.1685])
+def test_refinement_step_is_a_64_bit_quotient(psi):
+    """One Gauss-Newton step of a plane, far from its angle, against the same step in extended precision: 16
+    roundings of 2^-53 of the step (moments exact, about eight products and sums each in the numerator
+    and the divisor)."""
+    H, W = 33, 40
+    v, u = np.mgrid[0:H, 0:W]
+    l = (3 * v - u).astype(np.float32)
+    got = sgd.refine_roll(dev(l)[None], None, psi, 1).cpu().numpy()[0, 1, 0]
+    x = np.longdouble
+    uu, vv = u - x(W - 1) / 2, v - x(H - 1) / 2
+    m = lambda a, b: (a * b).sum() / x(H * W)
+    c, s = np.cos(x(psi)), np.sin(x(psi))
+    X, Y = uu * c + vv * s, vv * c - uu * s
+    a1 = m(Y, l.astype(x)) / m(Y, Y)
+    g, curv = a1 * (m(X, l.astype(x)) - a1 * m(X, Y)), a1 * a1 * (m(X, X) - m(X, Y) ** 2 / m(Y, Y))
+    want = x(psi) - g / curv
+    assert 1.0 < abs(float(g / curv)) and abs(float(want)) < math.pi / 2
+    assert abs(float(x(got) - want)) <= 16 * 2.0 ** -53 * abs(float(g / curv)) + 2.0 ** -53
