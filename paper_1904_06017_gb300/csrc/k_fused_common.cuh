@@ -80,6 +80,15 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity)
         : "memory");
     return ok != 0;
 }
+// The same for at most about a second (a millisecond under the stall test hook).
+__device__ __forceinline__ bool mbar_wait_limited(uint64_t *bar, uint32_t parity, bool stall)
+{
+    const long long limit = stall ? (1ll << 21) : (1ll << 31), t0 = clock64();
+    bool ok = false;
+    while (!(ok = mbar_try_wait(bar, parity)) && clock64() - t0 < limit) {
+    }
+    return ok;
+}
 
 __device__ __forceinline__ void tma_load_3d(void *dst, const CUtensorMap *map, int c0, int c1,
                                             int c2, uint64_t *bar)
@@ -152,13 +161,12 @@ __device__ __forceinline__ bool stage_images(const PairDesc *pd, const FusedArgs
             tma_load_3d(sref, &pd->tmap_ref, 0, (x0 + a.ref_box_x) / 16, y0, bar);
             tma_load_3d(stgt, &pd->tmap_tgt, 0, x0 / 16, y0, bar);
         }
-        const long long limit = stall ? (1ll << 21) : (1ll << 31);
-        const long long t0 = clock64();
-        bool ok = false;
-        while (!(ok = mbar_try_wait(bar, (uint32_t)(iter & 1))) && clock64() - t0 < limit) {
-        }
+        const bool ok = mbar_wait_limited(bar, (uint32_t)(iter & 1), stall);
         *flag = ok ? 1 : 0;
-        if (!ok) atomicOr(a.status, 1);
+        if (!ok) {
+            atomicOr(a.status, 1);
+            mbar_wait_limited(bar, (uint32_t)(iter & 1), stall);   // the CTA returns: no copy may land after it
+        }
     }
     __syncthreads();
     return *flag != 0;

@@ -411,20 +411,15 @@ k_march(const __grid_constant__ PairDesc single, const PairDesc *__restrict__ pa
             int kslot = 0, cslot = 0, islot = 0;   // (islot: the intensity and FP32 rings' slot of cost row cr)
             for (int p = 0; p < nsteps + TAIL; ++p) {
                 int bad = 0;
+                bool issued = true;
                 if (p < nsteps) {
                     // ---- the step's rows: wait for their bytes, widen them, store the statistics
                     uint64_t *bar = &s_bar[(gbase + p) & 1];
                     const uint32_t parity = (uint32_t)((gbase + p) >> 1) & 1u;
-                    if (!mbar_try_wait(bar, parity)) {
-                        // bounded as in stage_images: a fail-safe that sets the status word
-                        const long long limit = a.stall_test ? (1ll << 21) : (1ll << 31), t0 = clock64();
-                        bool ok = false;
-                        while (!(ok = mbar_try_wait(bar, parity)) && clock64() - t0 < limit) {
-                        }
-                        if (!ok) {
-                            bad = 1;
-                            atomicOr(a.status, 1);
-                        }
+                    // bounded as in stage_images: a fail-safe that sets the status word
+                    if (!mbar_try_wait(bar, parity) && !mbar_wait_limited(bar, parity, a.stall_test != 0)) {
+                        bad = 1;
+                        atomicOr(a.status, 1);
                     }
                     {
                         const uint8_t *rp = raw + (((gbase + p) & 1) * 4 + lr) * rowb;
@@ -458,6 +453,7 @@ k_march(const __grid_constant__ PairDesc single, const PairDesc *__restrict__ pa
                     // (the bytes of group p have been read; after an expired wait the barrier's phase is
                     // still open and must not be armed again: the CTA returns at the end of this step)
                     if (tid == 0 && !bad) issue(p + 2);
+                    issued = !bad;
                     load_stats(p + 1);
                     // intensities of the step's cost rows: image row cr + rw of the segment
                     {
@@ -524,7 +520,19 @@ k_march(const __grid_constant__ PairDesc single, const PairDesc *__restrict__ pa
                         if (++islot == RS) islot = 0;
                     }
                 }
-                if (__syncthreads_or(bad)) return;
+                if (__syncthreads_or(bad)) {
+                    // the CTA returns: no copy may land after it.  Thread 0 waits, with a limit too, for the
+                    // groups that it has armed: the next one, and this one or the one armed in its place
+                    if (tid == 0) {
+                        for (int gi = p + 1; gi >= p; --gi) {
+                            const int w = gi == p && issued ? p + 2 : gi;
+                            if (w < nsteps)
+                                mbar_wait_limited(&s_bar[(gbase + w) & 1], (uint32_t)((gbase + w) >> 1) & 1u,
+                                                  a.stall_test != 0);
+                        }
+                    }
+                    return;
+                }
             }
         } else if (!REF || warp < S::PW + kMarchCW) {
             // ------------------------------------------------------------------ consumers

@@ -282,13 +282,12 @@ __device__ __forceinline__ bool sc_stage(const PairDesc *pd, const FusedArgs &a,
                 tma_load_3d(stgt, &pd->tmap_tgt, 0, x0 / 16, y0, bar);
             }
         }
-        const long long limit = stall ? (1ll << 21) : (1ll << 31);
-        const long long t0 = clock64();
-        bool ok = false;
-        while (!(ok = mbar_try_wait(bar, (uint32_t)(iter & 1))) && clock64() - t0 < limit) {
-        }
+        const bool ok = mbar_wait_limited(bar, (uint32_t)(iter & 1), stall);
         *flag = ok ? 1 : 0;
-        if (!ok) atomicOr(a.status, 1);
+        if (!ok) {
+            atomicOr(a.status, 1);
+            mbar_wait_limited(bar, (uint32_t)(iter & 1), stall);   // the CTA returns: no copy may land after it
+        }
     }
     __syncthreads();
     return *flag != 0;
