@@ -15,8 +15,8 @@
 //   - has every disparity of a pixel in the registers of one quad, so the minimum, the candidate
 //     range or the winner follow without running state (one chunk);
 //   - splits into as many row segments as fill the SMs, whatever the frame size.
-// It is bound by instruction issue (60 % of the slots at N = 128; wait and math-pipe stalls), the
-// tensor pipe at 34 %.  1920 x 1080, D = 128, w = 9, k = 11: FP16 form 1.28 -> 0.69 ms; FP32 form
+// It is bound by shared memory and issue (FP32 form at N = 128: shared-memory pipe 71 %, issue slots 55 %,
+// tensor pipe 40 %; most stalls wait for a fixed latency or the math pipes).  1920 x 1080, D = 128, w = 9, k = 11: FP16 form 1.28 -> 0.69 ms; FP32 form
 // with k_refine 1.34 -> 0.83 ms (0.60 + 0.23).  D = 192, k = 13, FP16 (two passes of 96): 1.80 ->
 // 1.19 ms.
 //
@@ -60,7 +60,7 @@ namespace sgb {
 // stay in a second ring), kMarchPlain (FP16 / BF16 storage: the running WTA on the 16-bit sums and
 // the step's outputs).
 constexpr int kMarchScreen = 0, kMarchRefine = 1, kMarchPlain = 2;
-constexpr int kMarchUnroll = 16, kMarchUnroll32 = 16;
+constexpr int kMarchUnroll = 16;
 constexpr int kMarchRows = 2;
 constexpr int kMarchCW = 8;         // consumer warps: the eight patches of a band
 constexpr int kMarchRW = 8;         // refiner warps: four for the rows of a band, four for its ambiguous pixels
@@ -244,6 +244,15 @@ __device__ __forceinline__ void march_eval3(const float *ring32, const float *sI
     }
 }
 
+// The end of a CTA that gave up on a copy: no copy may land after it, so the row groups g0 and g1 (of
+// `end`) that it has in flight are waited for, with a limit too.  (A call: inlined, its registers cost
+// the loop of some instantiations up to 3 %.)
+static __device__ __noinline__ void march_drain(uint64_t *bar, int g0, int g1, int end, bool stall)
+{
+    if (g0 < end) mbar_wait_limited(bar + (g0 & 1), (uint32_t)(g0 >> 1) & 1u, stall);
+    if (g1 < end) mbar_wait_limited(bar + (g1 & 1), (uint32_t)(g1 >> 1) & 1u, stall);
+}
+
 // One CTA per work item: item blockIdx.x of one frame's strips and segments, or of a batch's list.
 template <int RB, int N, int MODE, typename T>
 __global__ void __launch_bounds__((MarchShape<RB, N>::threads(MODE)), march_ctas(N, MODE != kMarchPlain))
@@ -411,15 +420,20 @@ k_march(const __grid_constant__ PairDesc single, const PairDesc *__restrict__ pa
             int kslot = 0, cslot = 0, islot = 0;   // (islot: the intensity and FP32 rings' slot of cost row cr)
             for (int p = 0; p < nsteps + TAIL; ++p) {
                 int bad = 0;
-                bool issued = true;
                 if (p < nsteps) {
                     // ---- the step's rows: wait for their bytes, widen them, store the statistics
                     uint64_t *bar = &s_bar[(gbase + p) & 1];
                     const uint32_t parity = (uint32_t)((gbase + p) >> 1) & 1u;
-                    // bounded as in stage_images: a fail-safe that sets the status word
-                    if (!mbar_try_wait(bar, parity) && !mbar_wait_limited(bar, parity, a.stall_test != 0)) {
-                        bad = 1;
-                        atomicOr(a.status, 1);
+                    if (!mbar_try_wait(bar, parity)) {
+                        // bounded as in stage_images: a fail-safe that sets the status word
+                        const long long limit = a.stall_test ? (1ll << 21) : (1ll << 31), t0 = clock64();
+                        bool ok = false;
+                        while (!(ok = mbar_try_wait(bar, parity)) && clock64() - t0 < limit) {
+                        }
+                        if (!ok) {
+                            bad = 1;
+                            atomicOr(a.status, 1);
+                        }
                     }
                     {
                         const uint8_t *rp = raw + (((gbase + p) & 1) * 4 + lr) * rowb;
@@ -453,7 +467,6 @@ k_march(const __grid_constant__ PairDesc single, const PairDesc *__restrict__ pa
                     // (the bytes of group p have been read; after an expired wait the barrier's phase is
                     // still open and must not be armed again: the CTA returns at the end of this step)
                     if (tid == 0 && !bad) issue(p + 2);
-                    issued = !bad;
                     load_stats(p + 1);
                     // intensities of the step's cost rows: image row cr + rw of the segment
                     {
@@ -521,16 +534,8 @@ k_march(const __grid_constant__ PairDesc single, const PairDesc *__restrict__ pa
                     }
                 }
                 if (__syncthreads_or(bad)) {
-                    // the CTA returns: no copy may land after it.  Thread 0 waits, with a limit too, for the
-                    // groups that it has armed: the next one, and this one or the one armed in its place
-                    if (tid == 0) {
-                        for (int gi = p + 1; gi >= p; --gi) {
-                            const int w = gi == p && issued ? p + 2 : gi;
-                            if (w < nsteps)
-                                mbar_wait_limited(&s_bar[(gbase + w) & 1], (uint32_t)((gbase + w) >> 1) & 1u,
-                                                  a.stall_test != 0);
-                        }
-                    }
+                    // thread 0 has armed the next group, and this one or, had it landed, its successor
+                    if (tid == 0) march_drain(s_bar, gbase + p + 1, gbase + p + (bad ? 0 : 2), gbase + nsteps, a.stall_test != 0);
                     return;
                 }
             }
@@ -565,7 +570,7 @@ k_march(const __grid_constant__ PairDesc single, const PairDesc *__restrict__ pa
                     for (int nbk = 0; nbk < N / 8; ++nbk)
 #pragma unroll
                         for (int k = 0; k < 4; ++k) acc[nbk][k] = 0.f;
-#pragma unroll (N == 32 ? kMarchUnroll32 : kMarchUnroll)
+#pragma unroll kMarchUnroll
                     for (int r = 0; r < NKS; ++r) {
                         const float *irow = sI + isl * kMarchSI + px0 + 2 * t4;
                         const float2 qlo = *reinterpret_cast<const float2 *>(irow);
