@@ -31,10 +31,10 @@ WORKLOAD = "road-stereo 1920x1080 D=128 w=9 k=11 sigma0=3 sigma1=10, warp + fuse
 SM_COUNT_GB300 = 152
 FP32_LANES_PER_SM = 128
 SM_MAX_MHZ = 2070.0
-# DRAM traffic of one fused-kernel launch on this workload, from the ncu capture summarised
+# DRAM traffic of one fused step (k_march and k_refine) on this workload, from the ncu capture summarised
 # in profiles/ (dram__bytes_read.sum + dram__bytes_write.sum); valid only for the kernel
 # source with this SHA-256 prefix.
-FUSED_TRAFFIC = {"sha256": "972b7216c2da1f86", "bytes": 39214848}
+FUSED_TRAFFIC = {"sha256": "f78a67a9632a6650", "bytes": 87897088}
 FUSED_SOURCES = ("internal.cuh", "k_fused_common.cuh", "k_cost.cuh", "k_fused_tc.cuh", "k_sc_refine.cuh",
                  "k_march.cuh", "k_march_128.cu", "k_refine.cuh", "k_refine.cu")
 
@@ -716,6 +716,8 @@ def run_ours(args):
             "flops_per_launch": agg_flops, "flops_per_pixel_disparity": flops_per_unit,
             "avg_launch_ms": fused_avg_ms, "launches": n_fused,
             "peak_basis": "152 SMs x 128 FP32 lanes x 2 flop x 2070 MHz (nominal, derived)",
+            "note": "achieved counts the method's FP32 flops (a plain FP32 kernel's); the screening does most of them "
+                    "on the tensor cores, so frac compares with the FP32 pipe and is no utilisation (it can pass 1)",
             "fp32_probe_tflops": {"scalar_fma": probe_s / 1e3, "packed_f32x2_fma": probe_p / 1e3},
             "fused_gpix_disp_per_s": W * H * D / (fused_avg_ms * 1e-3) / 1e9}
     # the FP16 / BF16 forms do the same algorithmic work: their share of the same FP32 roofline
@@ -733,7 +735,7 @@ def run_ours(args):
             "tflops": t_tf, "peak": peaks.get("bf16_tflops"), "unit": "TFLOP/s",
             "frac": t_tf / peaks["bf16_tflops"] if peaks.get("bf16_tflops") else None,
             "peak_basis": "measured dense bf16 (same rate for fp16), MEASURED_PEAKS.json",
-            "note": "the form is bound by instruction issue (costs and weights), not the tensor pipe"}
+            "note": "the form is bound by shared memory and issue (costs and weights), not the tensor pipe"}
     variants["kernel"] = {"f32": "k_march + k_refine (screened FP32 form; the default)",
                           "f32_simt": "k_fused (the SIMT FP32 form: FP32 weights and accumulators on the CUDA cores)",
                           "f16": "k_march, plain mode (tensor-core aggregation of the FP16 costs, FP32 accumulators)",

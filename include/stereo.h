@@ -108,6 +108,10 @@ int stereo_params_default(stereo_params *p);
 /* Validate *p and create a context on the current CUDA device.  The context owns
  * padded image staging buffers, window statistics, tensor maps and the small
  * scratch of the disparity transformation (all allocated here, none later).
+ * Beside the padded images (1 byte per position each) and statistics (8 each), the
+ * tensor form up to bil = 13 holds per pixel: FP32 storage, 4 bytes where max_disp > 32
+ * and 4 more where the range takes several passes (max_disp > 128, or > 96 at bil = 13);
+ * FP16 / BF16 storage, 24 where it takes several passes.
  * Errors: STEREO_EINVAL for bad parameters, STEREO_ENOMEM, STEREO_ECUDA. */
 int stereo_create(const stereo_params *p, stereo_ctx **out);
 

@@ -69,6 +69,17 @@ __host__ __device__ constexpr int march_split(int rb, int D)
     const int full = (D - 1) / march_most(rb) * march_most(rb);
     return full > 0 && full + march_n(rb, D - full) < march_chunks(rb, D) * march_n(rb, D) ? full : 0;
 }
+// Rows of a k_refine tile on a frame of n 32 x 36 tiles.  36 where the tiles fill the SMs several times
+// over: the halo rows of the costs cost 1.3 times the rows at k = 11, 1.9 times at 12 rows (1024 x 768,
+// D = 96: 437 us the calls of a frame, 464 with 12 rows).  12 up to three tiles per SM, where the time is
+// that of the few tiles with the widest union of candidate ranges, those at the left border, or of a last
+// wave that is nearly empty (the calls of a frame back to back on one stream, host included, w = 9, k = 11
+// where not said: 320 x 240, D = 64: 210 -> 147 us; 588 x 385, D = 147, w = 11, k = 9: 373 -> 295; 640 x 480,
+// D = 64: 223 -> 214; 838 x 513, D = 137, w = k = 7: 425 -> 358; 960 x 540, D = 64: 278 -> 274).  Two CTAs per SM (80 registers a thread, which spill from k = 9 on)
+// but where the tiles are few and it spills (320 x 240: 147 against 161; 640 x 480: 221 against 214).
+constexpr int kRefineRows = 12;
+constexpr int refine_rows(int n, int nsm) { return n <= 3 * nsm ? kRefineRows : 36; }
+constexpr int refine_ctas(int n, int nsm, int rb) { return n <= 3 * nsm && (rb < 4 || 2 * n > 3 * nsm) ? 2 : 1; }
 // How a frame of FP32 storage runs (times of stereo_cost_aggregate_wta, w = 9, k = 11 where not said):
 //   kRouteTile    k_fused_sc, screening and refinement of a 32 x 36 tile in one kernel: ranges of at
 //                 most 32, where the screening is one chunk and the refinement most of the work
@@ -80,17 +91,6 @@ __host__ __device__ constexpr int march_split(int rb, int D)
 //                 kRouteSmall pixels, where the tiles are fewer than the SMs and a tile's latency is
 //                 the time (160 x 120, k = 13: 42 us against 85; 320 x 240, k = 9: 54 against 77; but
 //                 400 x 300, D = 30: 93 against 87, its refiners are slower where many candidates tie)
-// Rows of a k_refine tile on a frame of n 32 x 36 tiles.  36 where the tiles fill the SMs several times
-// over: the halo rows of the costs cost 1.3 times the rows at k = 11, 1.9 times at 12 rows (1024 x 768,
-// D = 96: 437 us the calls of a frame, 464 with 12 rows).  12 up to three tiles per SM, where the time is
-// that of the few tiles with the widest union of candidate ranges, those at the left border, or of a last
-// wave that is nearly empty (w = 9, k = 11 where not said: 320 x 240, D = 64: 210 -> 147 us; 588 x 385,
-// D = 147, w = 11, k = 9: 373 -> 295; 640 x 480, D = 64: 223 -> 214; 838 x 513, D = 137, w = k = 7: 425 ->
-// 358; 960 x 540, D = 64: 278 -> 274).  Two CTAs per SM (80 registers a thread, which spill from k = 9 on)
-// but where the tiles are few and it spills (320 x 240: 147 against 161; 640 x 480: 221 against 214).
-constexpr int kRefineRows = 12;
-constexpr int refine_rows(int n, int nsm) { return n <= 3 * nsm ? kRefineRows : 36; }
-constexpr int refine_ctas(int n, int nsm, int rb) { return n <= 3 * nsm && (rb < 4 || 2 * n > 3 * nsm) ? 2 : 1; }
 enum { kRouteTile = 0, kRouteMarch = 1, kRouteRefine = 2 };
 constexpr int kRouteSmall = 81920;
 __host__ __device__ constexpr int sc_route(int W, int H, int D)
