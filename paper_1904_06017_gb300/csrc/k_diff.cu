@@ -806,17 +806,31 @@ struct CbArgs {
 
 // The constants that are subtracted from the reference values and means (x) and the target's
 // (y): both adjoints depend only on differences t - mu_b and r - mu_a, which are here formed
-// after sums over d, so the images' common level is taken off first.  The median of three
-// pixels (0 where it is not finite).
-__device__ __forceinline__ float median3(float a, float b, float c)
+// after sums over d, so the images' common level is taken off first.  Of five pixels, the middle
+// between the second lowest and the second highest (0 where it is not finite): half way between the
+// levels of an image that has two, and no single pixel sets it.
+__device__ __forceinline__ float cb_level(const float *img, int W, int H)
 {
-    const float m = fmaxf(fminf(a, b), fminf(fmaxf(a, b), c));
+    float v[5];
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+        const int y = k == 0 ? H / 2 : k < 3 ? H / 4 : 3 * H / 4, x = k == 0 ? W / 2 : k & 1 ? W / 4 : 3 * W / 4;
+        v[k] = img[(size_t)y * W + x];
+    }
+    float lo = INFINITY, lo2 = INFINITY, hi = -INFINITY, hi2 = -INFINITY;
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+        lo2 = fminf(lo2, fmaxf(lo, v[k]));
+        lo = fminf(lo, v[k]);
+        hi2 = fmaxf(hi2, fminf(hi, v[k]));
+        hi = fmaxf(hi, v[k]);
+    }
+    const float m = 0.5f * lo2 + 0.5f * hi2;
     return isfinite(m) ? m : 0.f;
 }
 __device__ __forceinline__ float2 cb_levels(const float *ref, const float *tw, int W, int H)
 {
-    const size_t p0 = (size_t)(H / 2) * W + W / 2, p1 = (size_t)(H / 4) * W + W / 4, p2 = (size_t)(3 * H / 4) * W + 3 * W / 4;
-    return make_float2(median3(ref[p0], ref[p1], ref[p2]), median3(tw[p0], tw[p1], tw[p2]));
+    return make_float2(cb_level(ref, W, H), cb_level(tw, W, H));
 }
 
 // Extended reference positions X in [-rw, W-1+rw] x [-rw, H-1+rw], a 32 x cb_ty tile per block

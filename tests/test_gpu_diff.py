@@ -543,3 +543,24 @@ def test_refinement_step_is_a_64_bit_quotient(psi):
     want = x(psi) - g / curv
     assert 1.0 < abs(float(g / curv)) and abs(float(want)) < math.pi / 2
     assert abs(float(x(got) - want)) <= 16 * 2.0 ** -53 * abs(float(g / curv)) + 2.0 ** -53
+
+
+@pytest.mark.parametrize("axis", [0, 1])
+def test_gradients_of_an_image_of_two_levels(axis):
+    """Low contrast (+-1, a standard deviation of 0.58) on two levels, 20 and 240: the gradients are
+    differences of sums of values up to 110 from the middle, each rounded at 2^-24: four such roundings
+    of the contrast, as the root mean square over eight pairs (geometric mean; the target's, which a level
+    taken from one half doubles)."""
+    W, H, D = 96, 64, 24
+    x = np.arange(W) < W // 2 if axis else (np.arange(H) < H // 2)[:, None]
+    level = np.where(x, 20.0, 240.0) * np.ones((H, W))
+    err = []
+    for seed in range(8):
+        rng = np.random.default_rng(seed)
+        ref, tgt = [(level + rng.uniform(-1, 1, (H, W))).astype(np.float32).astype(np.float64) for _ in range(2)]
+        sh, gl = np.zeros(H, np.float32), rng.normal(size=(H, W)).astype(np.float32)
+        l, p, rts, ws = gpu_forward([ref], [tgt], [sh], D, 5, 11)
+        _, _, gto = odiff.disparity_vjp(ref, tgt, sh, D, 5, 11, S0, S1, T, gl.astype(np.float64))
+        _, gt = gpu_backward(p, rts, ws, gl[None])
+        err.append(np.sqrt(((gt[0] - gto) ** 2).mean() / (gto ** 2).mean()))
+    assert np.exp(np.log(err).mean()) <= 4 * 2.0 ** -24 * 110 / 0.58, err
